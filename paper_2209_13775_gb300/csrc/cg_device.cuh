@@ -2,6 +2,7 @@
 // largest eigenvalue of the Cauchy-Green tensor (Eq. 1; Sec. 2 "Cauchy-Green"), shared by
 // the regular pass (cg_ftle.cu) and the early evaluation (early_cg.cu).
 #pragma once
+#include "dfloat_device.cuh"
 #include "lcs_internal.cuh"
 
 #include <math.h>
@@ -27,23 +28,36 @@ __device__ __forceinline__ long long lattice_nbr(const CgLaunch &L, const long l
     return c[0] + (long long)L.n[0] * (c[1] + (long long)L.n[1] * c[2]);
 }
 
-// RN(x / d) for a fixed divisor d with y = RN(1 / d): q = RN(x y) is within about one
-// ulp of x / d, one FMA-corrected step q1 = RN(q + RN(x - q d) y) makes it faithful, so
-// the remainder x - q1 d is exact, and then RN(q1 + (x - q1 d) y) is the correctly
-// rounded quotient (Markstein 1990, Theorem 8: a faithful quotient corrected with the
-// correctly rounded reciprocal).  No overflow or underflow occurs for lattice spacings
-// and flow-map differences.
-__device__ __forceinline__ double div_fixed(double x, double d, double y)
+// RN(x / d) for a fixed divisor d.  FP64 issue limits this pass, so the divisor's quotient takes two
+// operations where launch_cg's exhaustive check of the divisor (fixed_divisor_exact) allows it: with
+// y + yl = 1/d to 105 bits, yl <= 0, RN(x y + RN(x yl)) is the correctly rounded quotient unless x/d
+// lies within about 2^-104 of a midpoint of two FP64 values (Brisebarre & Muller 2008).  Otherwise
+// with y = RN(1 / d) alone: q = RN(x y) is within about one ulp of x / d, one FMA-corrected step
+// makes it faithful, so the remainder x - q1 d is exact, and RN(q1 + (x - q1 d) y) is the correctly
+// rounded quotient (Markstein 1990, Theorem 8).  No overflow or underflow occurs for lattice
+// spacings and flow-map differences.  An infinite x gives NaN either way (yl <= 0).
+__device__ __forceinline__ double div_fixed(const CgLaunch &L, int b, double x)
 {
-    const double q = __dmul_rn(x, y);
+    const double y = L.rh2[b];
+    if (L.div2) return __fma_rn(x, y, __dmul_rn(x, L.rl2[b]));
+    const double d = L.h2[b], q = __dmul_rn(x, y);
     const double q1 = __fma_rn(__fma_rn(-q, d, x), y, q);
     return __fma_rn(__fma_rn(-q1, d, x), y, q1);
+}
+
+// (double)x without the FP64 pipe's conversion (which issues at the FP64 rate) for a normal x
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned u = __float_as_uint(x), e = u & 0x7f800000u;
+    if (e - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+    return (double)x;
 }
 
 // neighbour position with the periodic shift of axis b (a == b only; w in {-1, 0, 1})
 __device__ __forceinline__ double nbr_pos(float x, int w, double sh, bool shifted)
 {
-    double v = (double)x;
+    double v = widen(x);
     if (shifted && w != 0) v = __dadd_rn(v, w > 0 ? sh : -sh);
     return v;
 }
@@ -204,4 +218,146 @@ __device__ __forceinline__ double eig_max3(const double *C)
         beta -= f * (double)__frcp_rn((float)fp);
     }
     return (q + p * beta) * is;
+}
+
+// ------------------------------------------------------- differences and FTLE
+
+// one axis of a seed's differences: mode 1 central (F1 - F2) / 2h, 2 forward (-3 F0 + 4 F1 - F2) / 2h,
+// 3 backward (3 F0 - 4 F1 + F2) / 2h, 0 none (NaN); w1, w2: periods crossed by the two other points
+struct AxisDiff {
+    int mode, w1, w2;
+};
+
+// the quotient in FP64: every operation round-to-nearest, none contracted (the plain definition's bits)
+__device__ __forceinline__ double axis_grad64(const CgLaunch &L, int b, const AxisDiff &d, bool on, float f0, float f1,
+                                              float f2)
+{
+    if (d.mode == 0) return __longlong_as_double(0x7ff8000000000000LL);
+    const double sh = L.period[b], F1 = nbr_pos(f1, d.w1, sh, on), F2 = nbr_pos(f2, d.w2, sh, on);
+    double x;
+    if (d.mode == 1) {
+        x = __dsub_rn(F1, F2);
+    } else {
+        const double F0 = widen(f0);
+        x = d.mode == 2 ? __dsub_rn(__dadd_rn(__dmul_rn(-3.0, F0), __dmul_rn(4.0, F1)), F2)
+                        : __dadd_rn(__dsub_rn(__dmul_rn(3.0, F0), __dmul_rn(4.0, F1)), F2);
+    }
+    return div_fixed(L, b, x);
+}
+
+// the same quotient in double-FP32: the differences of FP32 positions are exact there
+__device__ __forceinline__ dfl axis_grad32(const CgLaunch &L, int b, const AxisDiff &d, bool on, float f0, float f1,
+                                           float f2)
+{
+    if (d.mode == 0) return {__int_as_float(0x7fc00000), 0.0f};
+    dfl x;
+    int k = d.w1 - d.w2;
+    if (d.mode == 1) {
+        x = df_two_sum(f1, -f2);
+    } else {
+        x = df_add(df_add(df_two_prod(-3.0f, f0), 4.0f * f1), -f2);
+        k = 4 * d.w1 - d.w2;
+        if (d.mode == 3) {
+            x = df_neg(x);
+            k = -k;
+        }
+    }
+    if (on && k != 0) x = df_add(x, df_mul(dfl{L.psh[b], L.psl[b]}, (float)k));
+    return df_mul(x, dfl{L.rhf[b], L.rlf[b]});
+}
+
+// C = grad F^T grad F (Eq. 1) in FP64, packed upper triangle row by row, round-to-nearest products
+// and sums in the order of a
+template <int DIM>
+__device__ __forceinline__ void cauchy_green64(const double (*G)[DIM], double *C)
+{
+    int o = 0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+#pragma unroll
+        for (int j = i; j < DIM; ++j) {
+            // the sum starts from +0.0, which only matters for an off-diagonal sum of negative zeros
+            double s = __dmul_rn(G[0][i], G[0][j]);
+            if (i != j) s = __dadd_rn(0.0, s);
+#pragma unroll
+            for (int a = 1; a < DIM; ++a) s = __dadd_rn(s, __dmul_rn(G[a][i], G[a][j]));
+            C[o++] = s;
+        }
+}
+
+template <int DIM>
+static __device__ __noinline__ float ftle_from_c64(const double *C, float half_inv_T)
+{
+    return log_lambda(DIM == 2 ? eig_max2(C) : eig_max3(C)) * half_inv_T;
+}
+
+// sigma = ln(lambda_max(G^T G)) * half_inv_T with G in double-FP32 (its entries' magnitudes between
+// 2^-40 and 2^40 at the largest: nothing below then leaves the FP32 range)
+template <int DIM>
+__device__ __forceinline__ float ftle_from_grad32(const dfl (*G)[DIM], float half_inv_T)
+{
+    constexpr int NP = DIM == 2 ? 3 : 6;
+    dfl C[NP];
+    int o = 0;
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+#pragma unroll
+        for (int j = i; j < DIM; ++j) {
+            dfl s = df_mul(G[0][i], G[0][j]);
+#pragma unroll
+            for (int a = 1; a < DIM; ++a) s = df_add(s, df_mul(G[a][i], G[a][j]));
+            C[o++] = s;
+        }
+    if constexpr (DIM == 2) {
+        return df_log(df_eig_max2(C)) * half_inv_T;
+    } else {
+        bool ok;
+        const dfl lm = df_eig_max3(C, &ok);
+        if (ok) return df_log(lm) * half_inv_T;
+        double Cd[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) Cd[q] = df_to_double(C[q]);
+        return ftle_from_c64<3>(Cd, half_inv_T);
+    }
+}
+
+// whether G's largest entry lies where ftle_from_grad32 is safe (false for NaN and infinite entries)
+template <int DIM>
+__device__ __forceinline__ bool grad32_in_range(const dfl (*G)[DIM])
+{
+    float m = 0.0f;
+    bool nan = false;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a)
+#pragma unroll
+        for (int b = 0; b < DIM; ++b) {
+            m = fmaxf(m, fabsf(G[a][b].h));
+            nan |= isnan(G[a][b].h);
+        }
+    return !nan && m >= 0x1p-40f && m <= 0x1p40f;
+}
+
+// FTLE of a seed from its positions f[b][k][a] (axis b, point k = 0 the seed, 1 and 2 the two others,
+// component a) in double-FP32, in FP64 where grad F lies outside the safe range
+template <int DIM>
+__device__ __forceinline__ float ftle_from_positions(const CgLaunch &L, const AxisDiff *d, const float *f0,
+                                                     const float (*f1)[DIM], const float (*f2)[DIM], float half_inv_T)
+{
+    dfl G[DIM][DIM];
+#pragma unroll
+    for (int b = 0; b < DIM; ++b)
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) G[a][b] = axis_grad32(L, b, d[b], a == b, f0[a], f1[b][a], f2[b][a]);
+    bool none = false;   // an axis without differences: NaN whatever the others hold
+#pragma unroll
+    for (int b = 0; b < DIM; ++b) none |= d[b].mode == 0;
+    if (none) return __int_as_float(0x7fc00000);
+    if (L.df_ok && grad32_in_range<DIM>(G)) return ftle_from_grad32<DIM>(G, half_inv_T);
+    double G64[DIM][DIM], C[DIM == 2 ? 3 : 6];
+#pragma unroll
+    for (int b = 0; b < DIM; ++b)
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) G64[a][b] = axis_grad64(L, b, d[b], a == b, f0[a], f1[b][a], f2[b][a]);
+    cauchy_green64<DIM>(G64, C);
+    return ftle_from_c64<DIM>(C, half_inv_T);
 }

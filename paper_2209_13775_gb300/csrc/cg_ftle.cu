@@ -5,18 +5,21 @@
 // the eigenvalues of C; Sec. 1: the FTLE is derived from the largest one,
 // sigma = ln(sqrt(lambda_max)) / |T|.
 //
-// One thread per seed, FP64 from the FP32 flow map.  FP64 issue is the limit of this
-// kernel on GB300, so the FP64 work is kept to what the results need:
-//  * grad F and C: every difference, product and sum is a round-to-nearest operation
-//    without contraction, and the division by 2h is correctly rounded (Markstein's
-//    method below), so both equal the plain FP64 definition bit for bit;
-//  * lambda_max: 2x2 from the quadratic formula; 3x3 from the characteristic cubic of
-//    the shifted, scaled matrix (Smith 1961), whose trigonometric root is taken in FP32
-//    and polished by two FP64 Newton steps (relative error ~1e-15 for a simple root),
-//    and by Jacobi rotations where the two largest eigenvalues (nearly) coincide;
-//  * FTLE = ln(lambda_max) / (2 |T|) in FP32: log1p of the FP64 difference lambda_max - 1
-//    near 1, which keeps its relative accuracy (a few FP32 ulps) where sigma is near 0, and
-//    log of lambda_max elsewhere (log_lambda).
+// One thread per seed.  GB300 has two FP64 lanes per SM against 128 FP32 ones, so FP64 issue bounds
+// whatever stays in FP64 (ncu: the FP64 pipe 85% busy, issue 14%, when all of it did):
+//  * C, lambda_max and the eigenpairs, where asked for: every difference, product and sum of grad F and
+//    C is a round-to-nearest FP64 operation without contraction and the division by 2h is correctly
+//    rounded (div_fixed: two operations), so both equal the plain FP64 definition bit for bit.
+//    lambda_max: 2x2 from the quadratic formula; 3x3 from the characteristic cubic of the shifted,
+//    scaled matrix (Smith 1961), whose trigonometric root is taken in FP32 and polished by two FP64
+//    Newton steps, and by Jacobi rotations where the two largest eigenvalues (nearly) coincide;
+//  * the FTLE, an FP32 output: the same formulas in double-FP32 (dfloat_device.cuh), about 200 FP32
+//    operations per seed in 2D and 700 in 3D in place of 65 and 170 FP64 ones, whether or not C or
+//    lambda_max is asked for (one call's FTLE does not depend on its other outputs).  Auxiliary
+//    points keep FP64 (their divisor is another one at every seed).
+// Measured: 64 windows of 2048 x 1024 seeds, FTLE only, advection and differences 95.3 -> 79.7 ms (the
+// differences 17.6 -> 2.0); 256^3 seeds with C written, 6.0 -> 2.8 ms (57 FP64 operations per seed
+// left of 170: 1.5 ms of FP64 issue).
 #include "lcs_internal.cuh"
 
 #include <math.h>
@@ -50,8 +53,50 @@ __device__ __forceinline__ void aux_gradient(const CgLaunch &L, int job, long lo
 // variational grad F integrated with the flow map
 enum { GM_LATTICE = 0, GM_AUX = 1, GM_VAR = 2 };
 
-template <int DIM, bool EIG, int GM>
-__global__ void __launch_bounds__(256) cg_ftle_kernel(CgLaunch L)
+// The difference rule of axis b at lattice seed p (coordinate c along it, neighbours `stride` apart) and
+// the ids of its two other points: central, else forward, else backward, from seeds with status OK only.
+// The points two steps away are looked at only where the central difference does not exist.
+__device__ __forceinline__ AxisDiff axis_diff(const CgLaunch &L, const unsigned char *__restrict__ S, long long p, int c,
+                                              int b, long long stride, bool valid, long long *q1, long long *q2)
+{
+    const int n = L.n[b];
+    const bool per = L.periodic[b] != 0;
+    const long long span = stride * n;
+    AxisDiff d = {0, 0, 0};
+    *q1 = *q2 = p;
+    if (!valid) return d;
+    const int wp = per && c + 1 >= n ? 1 : 0, wm = per && c < 1 ? -1 : 0;
+    const long long p1 = p + stride - wp * span, m1 = p - stride - wm * span;
+    const bool okp = (per || c + 1 < n) && S[p1] == LCS_TRACER_OK, okm = (per || c >= 1) && S[m1] == LCS_TRACER_OK;
+    if (okp && okm) {
+        d = {1, wp, wm};
+        *q1 = p1;
+        *q2 = m1;
+        return d;
+    }
+    if (okp) {
+        const int w = per && c + 2 >= n ? 1 : 0;
+        const long long p2 = p + 2 * stride - w * span;
+        if ((per || c + 2 < n) && S[p2] == LCS_TRACER_OK) {
+            d = {2, wp, w};
+            *q1 = p1;
+            *q2 = p2;
+        }
+    } else if (okm) {
+        const int w = per && c < 2 ? -1 : 0;
+        const long long m2 = p - 2 * stride - w * span;
+        if ((per || c >= 2) && S[m2] == LCS_TRACER_OK) {
+            d = {3, wm, w};
+            *q1 = m1;
+            *q2 = m2;
+        }
+    }
+    return d;
+}
+
+// F64: C, lambda_max or eigenpairs wanted (EIG: the latter), so grad F and C are formed in FP64 as well
+template <int DIM, bool F64, bool EIG, int GM>
+__global__ void __launch_bounds__(256) cg_ftle_kernel(const __grid_constant__ CgLaunch L)
 {
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int jr = blockIdx.y;        // job relative to job0
@@ -59,93 +104,176 @@ __global__ void __launch_bounds__(256) cg_ftle_kernel(CgLaunch L)
     const long long N = L.N;
     if (p >= N) return;
     constexpr int NP = DIM == 2 ? 3 : 6;
+    const size_t out = (size_t)jr * N + p;
+    const float half_inv_T = L.ftle ? 0.5f / (float)L.absT[job] : 0.0f;   // sigma = ln(lambda) / (2 |T|)
     double G[DIM][DIM];
     if constexpr (GM == GM_AUX) {
         aux_gradient<DIM>(L, job, p, G);
     } else if constexpr (GM == GM_VAR) {
         const bool ok = L.status[(size_t)job * N + p] == LCS_TRACER_OK;
         const float *Mp = L.grad + ((size_t)job * N + p) * DIM * DIM;
+        float M[DIM][DIM];
 #pragma unroll
         for (int a = 0; a < DIM; ++a)
 #pragma unroll
-            for (int b = 0; b < DIM; ++b)
-                G[a][b] = ok ? (double)Mp[a * DIM + b] : __longlong_as_double(0x7ff8000000000000LL);
-    } else {
-    const float *X = L.xyz + (size_t)job * DIM * N;
-    const unsigned char *S = L.status + (size_t)job * N;
-    const long long idx[3] = {p % L.n[0], (p / L.n[0]) % L.n[1], DIM == 3 ? p / ((long long)L.n[0] * L.n[1]) : 0};
-    bool valid = S[p] == LCS_TRACER_OK;
+            for (int b = 0; b < DIM; ++b) M[a][b] = ok ? Mp[a * DIM + b] : __int_as_float(0x7fc00000);
+        if (!EIG && L.ftle) {
+            dfl Gf[DIM][DIM];
 #pragma unroll
-    for (int b = 0; b < DIM; ++b) {
-        int wp1, wm1, wp2, wm2;
-        long long qp1 = lattice_nbr(L, idx, b, 1, &wp1);
-        long long qm1 = lattice_nbr(L, idx, b, -1, &wm1);
-        long long qp2 = lattice_nbr(L, idx, b, 2, &wp2);
-        long long qm2 = lattice_nbr(L, idx, b, -2, &wm2);
-        bool okp1 = qp1 >= 0 && S[qp1] == LCS_TRACER_OK;
-        bool okm1 = qm1 >= 0 && S[qm1] == LCS_TRACER_OK;
-        bool okp2 = qp2 >= 0 && S[qp2] == LCS_TRACER_OK;
-        bool okm2 = qm2 >= 0 && S[qm2] == LCS_TRACER_OK;
-        int mode = !valid ? 0 : (okp1 && okm1) ? 1 : (okp1 && okp2) ? 2 : (okm1 && okm2) ? 3 : 0;
-        const double h2 = L.h2[b], rh2 = L.rh2[b], sh = L.period[b];
+            for (int a = 0; a < DIM; ++a)
 #pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-            const bool on = a == b;
-            const float *Xa = X + (size_t)a * N;
-            double d;
-            if (mode == 1) {
-                const double Fp1 = nbr_pos(Xa[qp1], wp1, sh, on), Fm1 = nbr_pos(Xa[qm1], wm1, sh, on);
-                d = div_fixed(__dsub_rn(Fp1, Fm1), h2, rh2);
-            } else if (mode == 2) {
-                const double F0 = (double)Xa[p];
-                const double Fp1 = nbr_pos(Xa[qp1], wp1, sh, on), Fp2 = nbr_pos(Xa[qp2], wp2, sh, on);
-                d = div_fixed(__dsub_rn(__dadd_rn(__dmul_rn(-3.0, F0), __dmul_rn(4.0, Fp1)), Fp2), h2, rh2);
-            } else if (mode == 3) {
-                const double F0 = (double)Xa[p];
-                const double Fm1 = nbr_pos(Xa[qm1], wm1, sh, on), Fm2 = nbr_pos(Xa[qm2], wm2, sh, on);
-                d = div_fixed(__dadd_rn(__dsub_rn(__dmul_rn(3.0, F0), __dmul_rn(4.0, Fm1)), Fm2), h2, rh2);
-            } else {
-                d = __longlong_as_double(0x7ff8000000000000LL);  // NaN
+                for (int b = 0; b < DIM; ++b) Gf[a][b] = {M[a][b], 0.0f};
+            float s = __int_as_float(0x7fc00000);
+            if (grad32_in_range<DIM>(Gf)) {
+                s = ftle_from_grad32<DIM>(Gf, half_inv_T);
+            } else if (ok) {
+                double C[NP];
+#pragma unroll
+                for (int a = 0; a < DIM; ++a)
+#pragma unroll
+                    for (int b = 0; b < DIM; ++b) G[a][b] = (double)M[a][b];
+                cauchy_green64<DIM>(G, C);
+                s = ftle_from_c64<DIM>(C, half_inv_T);
             }
-            G[a][b] = d;
+            L.ftle[out] = s;
+        }
+        if constexpr (F64) {
+#pragma unroll
+            for (int a = 0; a < DIM; ++a)
+#pragma unroll
+                for (int b = 0; b < DIM; ++b) G[a][b] = (double)M[a][b];
+        }
+    } else {
+        const float *X = L.xyz + (size_t)job * DIM * N;
+        const unsigned char *S = L.status + (size_t)job * N;
+        // lattice coordinates; 32-bit division where the ids fit (a 64-bit one is a long routine)
+        int c[3];
+        if (N <= 0x7fffffffLL) {
+            const unsigned u = (unsigned)p, r = u / (unsigned)L.n[0];
+            c[0] = (int)(u - r * (unsigned)L.n[0]);
+            c[2] = DIM == 3 ? (int)(r / (unsigned)L.n[1]) : 0;
+            c[1] = DIM == 3 ? (int)(r - (unsigned)c[2] * (unsigned)L.n[1]) : (int)r;
+        } else {
+            c[0] = (int)(p % L.n[0]);
+            c[1] = (int)((p / L.n[0]) % L.n[1]);
+            c[2] = DIM == 3 ? (int)(p / ((long long)L.n[0] * L.n[1])) : 0;
+        }
+        const bool valid = S[p] == LCS_TRACER_OK;
+        AxisDiff d[DIM];
+        float f0[DIM], f1[DIM][DIM], f2[DIM][DIM];
+        long long stride = 1;
+        bool sided = false;
+#pragma unroll
+        for (int b = 0; b < DIM; ++b) {
+            long long q1, q2;
+            d[b] = axis_diff(L, S, p, c[b], b, stride, valid, &q1, &q2);
+            stride *= L.n[b];
+            sided |= d[b].mode != 1;
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                f1[b][a] = X[(size_t)a * N + q1];
+                f2[b][a] = X[(size_t)a * N + q2];
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) f0[a] = sided ? X[(size_t)a * N + p] : 0.0f;
+        if (!EIG && L.ftle) L.ftle[out] = ftle_from_positions<DIM>(L, d, f0, f1, f2, half_inv_T);
+        if constexpr (F64) {
+#pragma unroll
+            for (int b = 0; b < DIM; ++b)
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) G[a][b] = axis_grad64(L, b, d[b], a == b, f0[a], f1[b][a], f2[b][a]);
         }
     }
-    }
-    // Eq. 1: C_ij = sum_a G_ai G_aj, packed upper triangle row by row
-    double C[NP];
-    int o = 0;
+    if constexpr (F64) {
+        double C[NP];
+        cauchy_green64<DIM>(G, C);
+        if (L.C) {
+            double *o = L.C + out * NP;
+            if (DIM == 3 && L.c16) {
 #pragma unroll
-    for (int i = 0; i < DIM; ++i)
+                for (int q = 0; q < NP; q += 2) *reinterpret_cast<double2 *>(o + q) = make_double2(C[q], C[q + 1]);
+            } else {
 #pragma unroll
-        for (int j = i; j < DIM; ++j) {
-            double s = 0.0;
-#pragma unroll
-            for (int a = 0; a < DIM; ++a) s = __dadd_rn(s, __dmul_rn(G[a][i], G[a][j]));
-            C[o++] = s;
+                for (int q = 0; q < NP; ++q) o[q] = C[q];
+            }
         }
-    const size_t out = (size_t)jr * N + p;
-    if (L.C) {
+        if constexpr (EIG) {   // lcs_cg_eigen
+            double ev[DIM], V[DIM * DIM];
+            eig_jacobi<DIM>(C, ev, V);
+            if (L.eigval) {
 #pragma unroll
-        for (int q = 0; q < NP; ++q) L.C[out * NP + q] = C[q];
-    }
-    if constexpr (EIG) {   // lcs_cg_eigen
-        double ev[DIM], V[DIM * DIM];
-        eig_jacobi<DIM>(C, ev, V);
-        if (L.eigval) {
+                for (int k = 0; k < DIM; ++k) L.eigval[out * DIM + k] = ev[k];
+            }
+            if (L.eigvec) {
 #pragma unroll
-            for (int k = 0; k < DIM; ++k) L.eigval[out * DIM + k] = ev[k];
+                for (int k = 0; k < DIM * DIM; ++k) L.eigvec[out * DIM * DIM + k] = V[k];
+            }
+        } else if (L.lam || (GM == GM_AUX && L.ftle)) {
+            const double lm = DIM == 2 ? eig_max2(C) : eig_max3(C);
+            if (L.lam) L.lam[out] = lm;
+            if (GM == GM_AUX && L.ftle) L.ftle[out] = log_lambda(lm) * half_inv_T;
         }
-        if (L.eigvec) {
-#pragma unroll
-            for (int k = 0; k < DIM * DIM; ++k) L.eigvec[out * DIM * DIM + k] = V[k];
-        }
-        return;
     }
-    if (L.lam || L.ftle) {
-        const double lm = DIM == 2 ? eig_max2(C) : eig_max3(C);
-        if (L.lam) L.lam[out] = lm;
-        // sigma = ln(sqrt(lm)) / |T| = ln(lm) / (2 |T|)
-        if (L.ftle) L.ftle[out] = log_lambda(lm) * (0.5f / (float)L.absT[job]);
+}
+
+// ------------------------------------------------------------------- launch
+
+bool fixed_divisor_exact(double d, double *y, double *yl)
+{
+    typedef unsigned __int128 u128;
+    typedef unsigned long long u64;
+    // 1/d = y + yl: yl from the exact remainder 1 - y d; y is the upper neighbour where the
+    // remainder is positive, so that yl <= 0
+    double yh = 1.0 / d, rem = fma(-yh, d, 1.0);
+    if (rem > 0.0) {
+        yh = nextafter(yh, INFINITY);
+        rem = fma(-yh, d, 1.0);
+    }
+    *y = yh;
+    *yl = rem / d;
+    if (rem == 0.0) return true;   // d a power of two
+    int e;
+    const u64 D = (u64)ldexp(frexp(d, &e), 53);   // significand, 2^52 <= D < 2^53
+    // |x y + RN(x yl) - x/d| < 2^-104 |x/d|: a wrong rounding needs a significand X of x with
+    // X 2^s - (2k + 1) D = r, |r| <= 16, s = 53 (X >= D) or 54 (X < D).  Every such X is tried.
+    int v = 0;
+    while (!((D >> v) & 1)) ++v;
+    const u64 m = D >> v;              // X is determined modulo the odd part of D
+    if (m < (1ULL << 46)) return v > 5;  // v > 5: no r qualifies; else more candidates than are worth trying
+    u64 inv = 1, half = (m + 1) / 2;     // 2^-(s - v - 1) mod m, from 1/2 mod m
+    for (int q = 0; q < 53 - v - 1; ++q) inv = (u64)((u128)inv * half % m);
+    for (int s = 53; s <= 54; ++s) {
+        if (s == 54) inv = (u64)((u128)inv * half % m);
+        for (int r = -16; r <= 16; ++r) {
+            // X 2^s = r + (2k + 1) D needs r = D (mod 2^(v+1)) (s > v): then X = ((r + D) / 2^(v+1)) 2^(v+1-s) mod m
+            const long long num = (long long)D + r;
+            if (r == 0 || num % (1LL << (v + 1))) continue;
+            const u64 x = (u64)((u128)((u64)num >> (v + 1)) * inv % m), lo = 1ULL << 52, hi = 1ULL << 53;
+            for (u64 X = x + (lo > x ? (lo - x + m - 1) / m * m : 0); X < hi; X += m) {
+                const double xd = (double)X;
+                if ((X >= D) == (s == 53) && fma(xd, yh, xd * *yl) != xd / d) return false;
+            }
+        }
+    }
+    return true;
+}
+
+void cg_prepare(CgLaunch &L)
+{
+    L.df_ok = 1;
+    for (int b = 0; b < 3; ++b) {
+        L.h2[b] = 2.0 * L.h[b];  // exact
+        if (!L.div2) {
+            L.rh2[b] = 1.0 / L.h2[b];
+            L.rl2[b] = 0.0;
+        }
+        const double r = 1.0 / L.h2[b];
+        L.rhf[b] = (float)r;
+        L.rlf[b] = (float)(r - (double)L.rhf[b]);
+        L.psh[b] = (float)L.period[b];
+        L.psl[b] = (float)(L.period[b] - (double)L.psh[b]);
+        if (b < L.dim && !(r >= 0x1p-60 && r <= 0x1p60 && fabs(L.period[b]) <= 0x1p60)) L.df_ok = 0;
     }
 }
 
@@ -153,16 +281,17 @@ cudaError_t launch_cg_ftle(const CgLaunch &L0, cudaStream_t s)
 {
     if (L0.N == 0 || L0.njobs == 0) return cudaSuccess;
     CgLaunch L = L0;
-    for (int b = 0; b < 3; ++b) {
-        L.h2[b] = 2.0 * L.h[b];  // exact
-        L.rh2[b] = 1.0 / L.h2[b];
-    }
-    int bt = 256;
+    cg_prepare(L);
+    L.c16 = (uintptr_t)L.C % 16 == 0;
+    const int bt = 256;
     dim3 grid((unsigned)((L.N + bt - 1) / bt), (unsigned)L.njobs);
     const bool eig = L.eigval || L.eigvec;
     const int gm = L.grad ? GM_VAR : (L.x0aux ? GM_AUX : GM_LATTICE);
-#define CG_LAUNCH(D, G) (eig ? cg_ftle_kernel<D, true, G><<<grid, bt, 0, s>>>(L) \
-                             : cg_ftle_kernel<D, false, G><<<grid, bt, 0, s>>>(L))
+    const bool f64 = L.C || L.lam || gm == GM_AUX;
+#define CG_LAUNCH(D, G)                                                   \
+    (eig ? cg_ftle_kernel<D, true, true, G><<<grid, bt, 0, s>>>(L)        \
+         : f64 ? cg_ftle_kernel<D, true, false, G><<<grid, bt, 0, s>>>(L) \
+               : cg_ftle_kernel<D, G == GM_AUX, false, G><<<grid, bt, 0, s>>>(L))
     if (L.dim == 2) {
         if (gm == GM_VAR) CG_LAUNCH(2, GM_VAR);
         else if (gm == GM_AUX) CG_LAUNCH(2, GM_AUX);

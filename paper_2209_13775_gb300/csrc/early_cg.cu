@@ -202,45 +202,23 @@ __global__ void early_fd_kernel(CgLaunch L, const int *__restrict__ cells0, cons
     const long long p = it.x;
     const long long idx[3] = {p % L.n[0], (p / L.n[0]) % L.n[1], DIM == 3 ? p / ((long long)L.n[0] * L.n[1]) : 0};
     const float *X = pos + (size_t)e * NM * DIM;
-    double G[DIM][DIM];
+    AxisDiff d[DIM];
+    float f0[DIM], f1[DIM][DIM], f2[DIM][DIM];
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) f0[a] = X[a];
 #pragma unroll
     for (int b = 0; b < DIM; ++b) {
-        int w1, w2;
-        const int mode = axis_mode(L, idx, b, cells0);
-        member(L, idx, 1 + 2 * b, mode, &w1);
-        member(L, idx, 2 + 2 * b, mode, &w2);
-        const double h2 = L.h2[b], rh2 = L.rh2[b], sh = L.period[b];
+        d[b].mode = axis_mode(L, idx, b, cells0);
+        member(L, idx, 1 + 2 * b, d[b].mode, &d[b].w1);
+        member(L, idx, 2 + 2 * b, d[b].mode, &d[b].w2);
 #pragma unroll
         for (int a = 0; a < DIM; ++a) {
-            const bool on = a == b;
-            const double F0 = (double)X[a];
-            const double F1 = nbr_pos(X[(1 + 2 * b) * DIM + a], w1, sh, on);
-            const double F2 = nbr_pos(X[(2 + 2 * b) * DIM + a], w2, sh, on);
-            double d;
-            if (mode == 1)
-                d = div_fixed(__dsub_rn(F1, F2), h2, rh2);
-            else if (mode == 2)
-                d = div_fixed(__dsub_rn(__dadd_rn(__dmul_rn(-3.0, F0), __dmul_rn(4.0, F1)), F2), h2, rh2);
-            else
-                d = div_fixed(__dadd_rn(__dsub_rn(__dmul_rn(3.0, F0), __dmul_rn(4.0, F1)), F2), h2, rh2);
-            G[a][b] = d;
+            f1[b][a] = X[(1 + 2 * b) * DIM + a];
+            f2[b][a] = X[(2 + 2 * b) * DIM + a];
         }
     }
-    constexpr int NP = DIM == 2 ? 3 : 6;
-    double C[NP];
-    int o = 0;
-#pragma unroll
-    for (int i = 0; i < DIM; ++i)
-#pragma unroll
-        for (int j = i; j < DIM; ++j) {
-            double s = 0.0;
-#pragma unroll
-            for (int a = 0; a < DIM; ++a) s = __dadd_rn(s, __dmul_rn(G[a][i], G[a][j]));
-            C[o++] = s;
-        }
-    const double lm = DIM == 2 ? eig_max2(C) : eig_max3(C);
-    // sigma = ln(sqrt(lm)) / (m |h|), as the regular pass forms it
-    ftle[p] = log_lambda(lm) * (0.5f / (float)((double)it.y * adt));
+    // sigma = ln(sqrt(lambda_max)) / (m |h|), as the regular pass forms it
+    ftle[p] = ftle_from_positions<DIM>(L, d, f0, f1, f2, 0.5f / (float)((double)it.y * adt));
 }
 
 }  // namespace
@@ -248,10 +226,7 @@ __global__ void early_fd_kernel(CgLaunch L, const int *__restrict__ cells0, cons
 cudaError_t launch_early_cg(const EarlyLaunch &E, cudaStream_t s)
 {
     CgLaunch L = E.cg;
-    for (int b = 0; b < 3; ++b) {
-        L.h2[b] = 2.0 * L.h[b];
-        L.rh2[b] = 1.0 / L.h2[b];
-    }
+    cg_prepare(L);
     const int bt = 256;
     const unsigned grid = (unsigned)((L.N + bt - 1) / bt);
     if (E.phase == 0) {

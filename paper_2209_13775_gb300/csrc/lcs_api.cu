@@ -649,6 +649,11 @@ extern "C" lcs_status lcs_seed_grid(lcs_ctx *ctx, const lcs_seed_desc *d, const 
             s->period[a] = 0.0;
         }
     }
+    s->div2 = 1;
+    for (int a = 0; a < s->dim; ++a) {
+        const double d = 2.0 * s->h[a];
+        if (!(d >= 1e-200 && d <= 1e200 && fixed_divisor_exact(d, &s->rh2[a], &s->rl2[a]))) s->div2 = 0;
+    }
     cudaError_t e = cudaMalloc(&s->d_xyz, sizeof(float) * s->dim * (size_t)N);
     if (e == cudaSuccess) e = launch_seed_grid(s->dim, s->n, s->lo, s->hi, s->periodic, N, s->d_xyz, ctx->stream);
     if (e == cudaSuccess && field && lcs_is_mesh(field)) {
@@ -1180,7 +1185,10 @@ static lcs_status cg_call(lcs_ctx *ctx, const lcs_flowmap *fm, int job, float *f
         L.periodic[a] = s->periodic[a];
         L.h[a] = s->h[a];
         L.period[a] = s->period[a];
+        L.rh2[a] = s->rh2[a];
+        L.rl2[a] = s->rl2[a];
     }
+    L.div2 = s->div2;
     L.N = (long long)N;
     L.job0 = j0;
     L.njobs = nj;
@@ -1318,7 +1326,10 @@ extern "C" lcs_status lcs_ftle_early(lcs_ctx *ctx, const lcs_field *f, const lcs
         L.periodic[a] = s->periodic[a];
         L.h[a] = s->h[a];
         L.period[a] = s->period[a];
+        L.rh2[a] = s->rh2[a];
+        L.rl2[a] = s->rl2[a];
     }
+    L.div2 = s->div2;
     L.N = fm->N;
     L.job0 = job;
     L.njobs = 1;

@@ -135,6 +135,8 @@ struct lcs_seeds {
     unsigned long long field_uid = 0;  // the tet field the cells refer to
     double h[3] = {1, 1, 1};           // lattice step per axis
     double period[3] = {0, 0, 0};      // hi - lo on periodic axes
+    double rh2[3] = {1, 1, 1}, rl2[3] = {0, 0, 0};  // 1 / (2 h) as two FP64 values, for quotients by 2 h in
+    int div2 = 0;                      //   two operations where every axis allows it (fixed_divisor_exact)
     long long aux_base_N = 0;          // > 0: auxiliary points of a lattice of that many seeds (lcs_seed_aux)
     double aux_delta[3] = {0, 0, 0};
 };
@@ -269,7 +271,14 @@ struct CgLaunch {
     int periodic[3];
     double h[3];
     double period[3];
-    double h2[3], rh2[3];        // 2 h and RN(1 / (2 h)), filled by launch_cg_ftle
+    double rh2[3], rl2[3];       // 1 / (2 h) as two FP64 values and whether div_fixed may use them (lcs_seeds)
+    int div2;
+    // filled by cg_prepare: 2 h, and in double-FP32 its reciprocal and the period (df_ok: both lie well
+    // inside the FP32 range)
+    double h2[3];
+    int df_ok;
+    int c16;                     // C is 16-byte aligned (set by launch_cg_ftle)
+    float rhf[3], rlf[3], psh[3], psl[3];
     long long N;
     int job0, njobs;
     const float *xyz;            // flow map base [njobs_total][dim][N]
@@ -287,6 +296,10 @@ struct CgLaunch {
 };
 
 cudaError_t launch_cg_ftle(const CgLaunch &L, cudaStream_t s);
+void cg_prepare(CgLaunch &L);
+// whether RN(x y + RN(x yl)) = RN(x / d) for every x of normal range, y + yl = 1/d with yl <= 0
+// (both written); d > 0 of normal range
+bool fixed_divisor_exact(double d, double *y, double *yl);
 
 // early Cauchy-Green evaluation (early_cg.cu): phase 0 scans the seeds of slot `job` (writes
 // t_eval and lists the early ones), phase 1 re-integrates the listed stencils and writes their FTLE
