@@ -117,9 +117,9 @@ template <int DIM, int ST>
 __global__ void __launch_bounds__(256) rk4_gather_kernel(RectParams P, const char *__restrict__ frames,
                                                          size_t fstride, Rk4Args A)
 {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long i = thread_tracer(A);
     int job = blockIdx.y;
-    if (i >= A.N) return;
+    if (i < 0) return;
     float x[DIM], cx[DIM];
     int img[DIM];
 #pragma unroll
@@ -224,9 +224,9 @@ template <int DIM, int ST>
 __global__ void __launch_bounds__(256) rk4_var_kernel(RectParams P, const char *__restrict__ frames, size_t fstride,
                                                       Rk4Args A)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long i = thread_tracer(A);
     const int job = blockIdx.y;
-    if (i >= A.N) return;
+    if (i < 0) return;
     float x[DIM], cx[DIM], M[DIM][DIM];
     int img[DIM];
 #pragma unroll
@@ -621,9 +621,9 @@ template <int PM>
 __global__ void __launch_bounds__(256) rk4_slice2d_kernel(RectParams P, const float4 *__restrict__ slices,
                                                           long long nodes, Slice2dOffsets O, Rk4Args A)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long i = thread_tracer(A);
     const int job = blockIdx.y;
-    if (i >= A.N) return;
+    if (i < 0) return;
     float x[2] = {A.seeds[i], A.seeds[A.N + i]}, cx[2] = {0.0f, 0.0f};
     int img[2] = {0, 0};
     wrap_periodic<2, PM>(P, x, cx, img);
@@ -689,7 +689,7 @@ static cudaError_t launch_slice2d(const RectParams &P, const lcs_field *f, const
                                                                       A.job_nsteps, O, nodes, slices);
     lcs_tm_end(L.ctx, 2, s);
     lcs_tm_begin(L.ctx, 0, s);
-    dim3 grid((unsigned)((A.N + bt - 1) / bt), (unsigned)L.njobs);
+    dim3 grid(seed_map_grid(A.map, A.N, bt), (unsigned)L.njobs);
     const int pm = P.periodic[0] | (P.periodic[1] << 1);
     if (pm == 0)
         rk4_slice2d_kernel<0><<<grid, bt, 0, s>>>(P, slices, nodes, O, A);
@@ -702,6 +702,27 @@ static cudaError_t launch_slice2d(const RectParams &P, const lcs_field *f, const
 }
 
 // ================================================================ dispatch
+
+SeedMap make_seed_map(int dim, const int *n, int bt)
+{
+    SeedMap M;
+    if ((dim != 2 && dim != 3) || bt % 32) return M;
+    const int e[3] = {dim == 2 ? 16 : 8, dim == 2 ? 16 : 8, 4};
+    long long seeds = 1, padded = 1, t[3] = {1, 1, 1};
+    for (int d = 0; d < dim; ++d) {
+        t[d] = ((long long)n[d] + e[d] - 1) / e[d];
+        seeds *= n[d];
+        padded *= t[d] * e[d];
+    }
+    if (padded * 4 > seeds * 5 || padded > 0x7fffffffLL) return M;
+    M.tiled = 1;
+    M.dim = dim;
+    for (int d = 0; d < dim; ++d) M.n[d] = n[d];
+    M.t0 = (unsigned)t[0];
+    M.t1 = (unsigned)t[1];
+    M.blocks8 = t[0] * t[1] * t[2];
+    return M;
+}
 
 RectParams make_rect_params(const lcs_field *f)
 {
@@ -727,7 +748,7 @@ template <int DIM, int ST>
 static cudaError_t launch_gather(const RectParams &P, const lcs_field *f, const Rk4Args &A, int njobs, int bt,
                                  cudaStream_t s)
 {
-    dim3 grid((unsigned)((A.N + bt - 1) / bt), (unsigned)njobs);
+    dim3 grid(seed_map_grid(A.map, A.N, bt), (unsigned)njobs);
     rk4_gather_kernel<DIM, ST><<<grid, bt, 0, s>>>(P, (const char *)f->d_frames, f->frame_stride, A);
     return cudaGetLastError();
 }
@@ -817,7 +838,8 @@ int launch_rk4_rect(lcs_ctx *ctx, const Rk4Launch &L, cudaStream_t s)
     }
     if (A.out_grad) {   // the variational equations elsewhere: their own one-pass kernel
         const int bt = L.block_threads > 0 && L.block_threads <= 256 ? L.block_threads : 256;
-        dim3 grid((unsigned)((A.N + bt - 1) / bt), (unsigned)L.njobs);
+        A.map = make_seed_map(L.lat_dim, L.lat_n, bt);
+        dim3 grid(seed_map_grid(A.map, A.N, bt), (unsigned)L.njobs);
         const char *fr = (const char *)f->d_frames;
         lcs_tm_begin(ctx, 0, s);
 #define VAR_LAUNCH(D, ST) rk4_var_kernel<D, ST><<<grid, bt, 0, s>>>(P, fr, f->frame_stride, A)
@@ -841,6 +863,7 @@ int launch_rk4_rect(lcs_ctx *ctx, const Rk4Launch &L, cudaStream_t s)
     }
     if (variant == 5) {
         int bt = L.block_threads > 0 && L.block_threads <= 256 ? L.block_threads : 256;
+        A.map = make_seed_map(L.lat_dim, L.lat_n, bt);
         e = launch_slice2d(P, f, A, L, bt, s);
         return e == cudaSuccess ? variant : -1;
     }
@@ -858,6 +881,7 @@ int launch_rk4_rect(lcs_ctx *ctx, const Rk4Launch &L, cudaStream_t s)
     } else {
         int bt = L.block_threads > 0 ? L.block_threads : 256;
         if (bt > 256) bt = 256;
+        A.map = make_seed_map(L.lat_dim, L.lat_n, bt);
         if (f->dim == 2) {
             if (f->storage == LCS_F32)
                 e = launch_gather<2, LCS_F32>(P, f, A, L.njobs, bt, s);

@@ -36,9 +36,9 @@ template <int ST>
 __global__ void __launch_bounds__(256) rk4_tet_kernel(TetDev T, Rk4Args A, const int *__restrict__ cells0,
                                                       unsigned *errword)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long i = thread_tracer(A);
     const int job = blockIdx.y;
-    if (i >= A.N) return;
+    if (i < 0) return;
     float x[3] = {A.seeds[i], A.seeds[A.N + i], A.seeds[2 * A.N + i]}, cx[3] = {0.0f, 0.0f, 0.0f};
     int cell = cells0[i];
     unsigned char st = LCS_TRACER_OK;
@@ -88,9 +88,9 @@ template <int ST>
 __global__ void __launch_bounds__(256) rk4_tri_kernel(TriDev T, Rk4Args A, const int *__restrict__ cells0,
                                                       unsigned *errword)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long i = thread_tracer(A);
     const int job = blockIdx.y;
-    if (i >= A.N) return;
+    if (i < 0) return;
     float x[2] = {A.seeds[i], A.seeds[A.N + i]}, cx[2] = {0.0f, 0.0f};
     int cell = cells0[i];
     unsigned char st = LCS_TRACER_OK;
@@ -145,9 +145,9 @@ template <int DIM, int ST, class MD>
 __global__ void __launch_bounds__(256) rk4_mesh_var_kernel(MD T, Rk4Args A, const int *__restrict__ cells0,
                                                            unsigned *errword)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long i = thread_tracer(A);
     const int job = blockIdx.y;
-    if (i >= A.N) return;
+    if (i < 0) return;
     float x[DIM], cx[DIM], M[DIM][DIM];
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
@@ -503,7 +503,8 @@ cudaError_t launch_rk4_tet(lcs_ctx *ctx, const Rk4Launch &L, const int *cells0, 
     A.out_grad = L.out_grad;
     if (L.N == 0) return cudaSuccess;
     const int bt = L.block_threads > 0 && L.block_threads <= 256 ? L.block_threads : 128;
-    dim3 grid((unsigned)((L.N + bt - 1) / bt), (unsigned)L.njobs);
+    A.map = make_seed_map(L.lat_dim, L.lat_n, bt);
+    dim3 grid(seed_map_grid(A.map, L.N, bt), (unsigned)L.njobs);
     if (A.out_grad) {   // the variational equations
         lcs_tm_begin(ctx, 0, s);
         if (f->kind == LCS_TRI) {

@@ -835,6 +835,10 @@ static lcs_status advect_rk4_rect(lcs_ctx *ctx, const lcs_field *f, const lcs_se
     L.host_snap_n = J.snap_n;
     L.snap_te = D.snap_te;
     L.work = want_work ? (char *)ctx->d_scratch + jb + sb : nullptr;
+    if (s->aux_base_N == 0) {
+        L.lat_dim = s->dim;
+        for (int a = 0; a < 3; ++a) L.lat_n[a] = s->n[a];
+    }
     if (o->wait_limit > 0.0) L.wait_ns = (unsigned long long)(o->wait_limit * 1e9);
     if (lcs_is_mesh(f)) {
         cudaError_t e = launch_rk4_tet(ctx, L, s->d_cells, o->walk_limit, ctx->stream);

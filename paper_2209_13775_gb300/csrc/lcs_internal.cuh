@@ -207,6 +207,27 @@ struct JobDev {
     float *snap_te = nullptr;  // [njobs][nsnap] end time t0 + T of each snapshot (a tracer still OK there)
 };
 
+// Which tracer a thread of a one-thread-per-tracer kernel integrates.  tiled: warps take 8 x 4 (2D) or
+// 4 x 4 x 2 (3D) blocks of the lattice and eight consecutive warps a 16 x 16 or 8 x 8 x 4 block, so that the
+// lanes of a warp start, and stay longer, in few cells (RK4 on the 1.6M-triangle stenosis, 4096 x 1024 seeds:
+// 31.7 -> 28.3 ms; on tets, 45 x 45 x 301 seeds: 3.27 -> 3.22 ms); otherwise thread t takes tracer t.
+struct SeedMap {
+    int tiled = 0, dim = 0;
+    int n[3] = {1, 1, 1};      // lattice
+    unsigned t0 = 1, t1 = 1;   // blocks of eight warps along x and y
+    long long blocks8 = 0;     // blocks of eight warps in all
+};
+
+// the map of a lattice of n seeds per axis for blocks of bt threads; linear where the padded lattice would
+// idle more than a fifth of the threads, or bt is no multiple of 32
+SeedMap make_seed_map(int dim, const int *n, int bt);
+
+static inline unsigned seed_map_grid(const SeedMap &M, long long N, int bt)
+{
+    const long long threads = M.tiled ? M.blocks8 * 256 : N;
+    return (unsigned)((threads + bt - 1) / bt);
+}
+
 struct Rk4Launch {
     lcs_ctx *ctx;
     const lcs_field *field;
@@ -238,6 +259,8 @@ struct Rk4Launch {
     const int *host_snap_n = nullptr;  // [nsnap] the same on the host
     const float *snap_te = nullptr;    // [njobs][nsnap] snapshot end times (device)
     unsigned long long wait_ns = LCS_WAIT_LIMIT_NS;  // ring kernels: bound on a wait for a frame copy
+    int lat_dim = 0;          // 2 or 3: the seeds are a lattice of lat_n per axis, x fastest; 0: any points
+    int lat_n[3] = {1, 1, 1};
 };
 
 // smallest seed count for which lcs_advect picks the re-bundled kernel by default

@@ -342,7 +342,33 @@ struct Rk4Args {
     const int *snap_n = nullptr;     // [nsnap] snapshot step counts (device; capped per job at use)
     const float *snap_te = nullptr;  // [njobs][nsnap] snapshot end times, the exit time of a tracer OK there
     unsigned long long wait_ns = LCS_WAIT_LIMIT_NS;  // ring kernels: bound on a wait for a frame copy
+    SeedMap map;                     // thread -> tracer of the one-thread-per-tracer kernels
 };
+
+// the calling thread's tracer (Rk4Args::map), or -1
+__device__ __forceinline__ long long thread_tracer(const Rk4Args &A)
+{
+    const SeedMap &M = A.map;
+    if (!M.tiled) {
+        const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+        return i < A.N ? i : -1;
+    }
+    const unsigned wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const unsigned b8 = wid >> 3, w = wid & 7;
+    if (b8 >= M.blocks8) return -1;
+    const unsigned r = b8 / M.t0, bx = b8 - r * M.t0;
+    if (M.dim == 2) {
+        const unsigned x = bx * 16 + (w & 1) * 8 + (lane & 7), y = r * 16 + (w >> 1) * 4 + (lane >> 3);
+        return x < (unsigned)M.n[0] && y < (unsigned)M.n[1] ? x + (long long)M.n[0] * y : -1;
+    }
+    const unsigned bz = r / M.t1, by = r - bz * M.t1;
+    const unsigned x = bx * 8 + (w & 1) * 4 + (lane & 3), y = by * 8 + ((w >> 1) & 1) * 4 + ((lane >> 2) & 3),
+                   z = bz * 4 + (w >> 2) * 2 + (lane >> 4);
+    return x < (unsigned)M.n[0] && y < (unsigned)M.n[1] && z < (unsigned)M.n[2]
+               ? x + (long long)M.n[0] * (y + (long long)M.n[1] * z)
+               : -1;
+}
+
 
 // Step after which snapshot s of a job with ns steps is taken.
 __device__ __forceinline__ int snap_step(const Rk4Args &A, int s, int ns) { return min(__ldg(A.snap_n + s), ns); }
