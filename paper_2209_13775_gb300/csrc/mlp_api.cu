@@ -27,65 +27,18 @@ extern "C" lcs_status lcs_gemm_bf16(lcs_ctx *ctx, long long M, int N, long long 
 
 namespace {
 
-// FP32 master parameters -> the inference block (canonical operand tiles + biases) and the
-// trainer's K-major BF16 operands and their transposes; one thread per destination element
-__global__ void mlp_refresh_kernel(const float *__restrict__ p, unsigned char *__restrict__ tiles,
-                                   __nv_bfloat16 *__restrict__ wk, __nv_bfloat16 *__restrict__ wt)
+// FP32 master parameters -> the operand tiles (their padding was zeroed when the network was made)
+__global__ void mlp_refresh_kernel(const float *__restrict__ p, unsigned char *__restrict__ tiles)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    // inference tiles: W0 (128 x 16), W1..W3 (128 x 128), W4 (16 x 128) as BF16 elements
-    const int n_w0 = 128 * 16, n_w = 128 * 128, n_w4 = 16 * 128;
-    const int n_tiles = n_w0 + 3 * n_w + n_w4;
-    const int n_k = n_tiles;                // trainer operands, same element counts
-    const int n_t = 3 * n_w + 128 * 16;     // transposes of W1..W3 and W4
-    if (i < n_tiles) {
-        int r, k, R, l;
-        uint32_t base;
-        float v;
-        if (i < n_w0) {
-            l = 0, R = 128, r = i / 16, k = i % 16, base = 0;
-            v = k < 7 ? p[MLP_OFF_W0 + r * 7 + k] : 0.0f;
-        } else if (i < n_w0 + 3 * n_w) {
-            const int j = i - n_w0;
-            l = 1 + j / n_w, R = 128, r = (j % n_w) / 128, k = j % 128, base = 4096 + 32768u * (l - 1);
-            v = p[MLP_OFF_W1 + (l - 1) * MLP_LAYER_STRIDE + r * 128 + k];
-        } else {
-            const int j = i - n_w0 - 3 * n_w;
-            l = 4, R = 16, r = j / 128, k = j % 128, base = 102400;
-            v = r < 3 ? p[MLP_OFF_W4 + r * 128 + k] : 0.0f;
-        }
-        const __nv_bfloat16 b = __float2bfloat16_rn(v);
-        *reinterpret_cast<__nv_bfloat16 *>(tiles + base + ckm_offset(R, r, k)) = b;
-        // trainer operand, row-major [out][in] with the same padding
-        wk[i] = b;
-        (void)l;
-    } else if (i < n_tiles + n_t) {
-        const int j = i - n_tiles;
-        if (j < 3 * n_w) {  // W_l^T [in][out]
-            const int l = 1 + j / n_w, in = (j % n_w) / 128, out = j % 128;
-            wt[j] = __float2bfloat16_rn(p[MLP_OFF_W1 + (l - 1) * MLP_LAYER_STRIDE + out * 128 + in]);
-        } else {            // W4^T [128 in][16 out]
-            const int q = j - 3 * n_w, in = q / 16, out = q % 16;
-            wt[j] = __float2bfloat16_rn(out < 3 ? p[MLP_OFF_W4 + out * 128 + in] : 0.0f);
-        }
-    } else if (i < n_tiles + n_t + 528) {
-        const int j = i - n_tiles - n_t;     // biases b0..b3, then b4 padded to 16
-        float v;
-        if (j < 512)
-            v = p[MLP_OFF_B0 + (j / 128) * MLP_LAYER_STRIDE + (j % 128)];
-        else
-            v = j - 512 < 3 ? p[MLP_OFF_B4 + (j - 512)] : 0.0f;
-        reinterpret_cast<float *>(tiles + 106496)[j] = v;
-    }
-    (void)n_k;
+    if (i < MLP_NPARAMS) mlp_store_param(tiles, i, p[i]);
 }
 
 }  // namespace
 
 cudaError_t launch_mlp_refresh(lcs_mlp *m, cudaStream_t s)
 {
-    const int total = (128 * 16 + 3 * 128 * 128 + 16 * 128) + (3 * 128 * 128 + 128 * 16) + 528;
-    mlp_refresh_kernel<<<(total + 255) / 256, 256, 0, s>>>(m->d_params, m->d_tiles, m->d_wk, m->d_wt);
+    mlp_refresh_kernel<<<(MLP_NPARAMS + 255) / 256, 256, 0, s>>>(m->d_params, m->d_tiles);
     return cudaGetLastError();
 }
 
@@ -114,8 +67,8 @@ extern "C" lcs_status lcs_mlp_create(lcs_ctx *ctx, const lcs_mlp_desc *d, const 
     if (e == cudaSuccess) e = cudaMalloc(&m->d_v, pb);
     if (e == cudaSuccess) e = cudaMalloc(&m->d_grad, pb);
     if (e == cudaSuccess) e = cudaMalloc(&m->d_tiles, MLP_TILE_BYTES);
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_wk, sizeof(__nv_bfloat16) * (128 * 16 + 3 * 128 * 128 + 16 * 128));
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_wt, sizeof(__nv_bfloat16) * (3 * 128 * 128 + 128 * 16));
+    if (e == cudaSuccess) e = cudaMalloc(&m->d_loss, sizeof(double));
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->d_tiles, 0, MLP_TILE_BYTES, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->d_m, 0, pb, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->d_v, 0, pb, ctx->stream);
     if (e == cudaSuccess)
@@ -167,8 +120,7 @@ extern "C" void lcs_mlp_free(lcs_mlp *m)
     cudaFree(m->d_v);
     cudaFree(m->d_grad);
     cudaFree(m->d_tiles);
-    cudaFree(m->d_wk);
-    cudaFree(m->d_wt);
+    cudaFree(m->d_loss);
     cudaFree(m->d_work);
     delete m;
 }
@@ -353,7 +305,6 @@ extern "C" lcs_status lcs_mlp_loss_grad(lcs_ctx *ctx, lcs_mlp *m, long long n, c
     LCS_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
     const float *dx = xyt, *dd = disp;
     float *tmp = nullptr;
-    double *dl = nullptr;
     if (!on_device) {
         LCS_CUDA_TRY(ctx, cudaMallocAsync((void **)&tmp, sizeof(float) * 5 * n, ctx->stream));
         LCS_CUDA_TRY(ctx, cudaMemcpyAsync(tmp, xyt, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, ctx->stream));
@@ -361,16 +312,15 @@ extern "C" lcs_status lcs_mlp_loss_grad(lcs_ctx *ctx, lcs_mlp *m, long long n, c
         dx = tmp;
         dd = tmp + 3 * n;
     }
-    LCS_CUDA_TRY(ctx, cudaMallocAsync((void **)&dl, sizeof(double), ctx->stream));
-    cudaError_t e = mlp_loss_grad(m, dx, n, dd, n, n, (float)rho_weight, ctx->num_sms, ctx->d_errword, dl, ctx->stream);
+    cudaError_t e = mlp_loss_grad(m, dx, n, dd, n, n, (float)rho_weight, ctx->num_sms, ctx->d_errword, m->d_loss,
+                                  ctx->stream);
     double lsum = 0.0;
     if (e == cudaSuccess && grads)
         e = cudaMemcpyAsync(grads, m->d_grad, sizeof(float) * MLP_NPARAMS,
                             on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess && loss) e = cudaMemcpyAsync(&lsum, dl, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess && loss) e = cudaMemcpyAsync(&lsum, m->d_loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess && loss) e = cudaStreamSynchronize(ctx->stream);
     if (tmp) cudaFreeAsync(tmp, ctx->stream);
-    cudaFreeAsync(dl, ctx->stream);
     if (e != cudaSuccess) return lcs_fail(ctx, LCS_ECUDA, "lcs_mlp_loss_grad: %s", cudaGetErrorString(e));
     if (loss) *loss = lsum / (double)n;
     if (!on_device) return lcs_synchronize(ctx);
@@ -432,7 +382,7 @@ extern "C" lcs_status lcs_surrogate_train(lcs_ctx *ctx, const lcs_field *f, lcs_
     }
     // integrator targets: RK4 displacement over tau from every sample
     cudaError_t e = mlp_targets(f, xyt, ns, (int)S, d->dt, disp, ctx->stream);
-    if (e == cudaSuccess) e = mlp_reserve(m, B, ctx->stream);
+    if (e == cudaSuccess) e = mlp_reserve(m, ctx->num_sms);
     for (long long it = 0; it < total && e == cudaSuccess; ++it) {
         const long long b = it % nb;
         e = mlp_loss_grad(m, xyt + b * B, ns, disp + b * B, ns, B, (float)d->rho_weight, ctx->num_sms, ctx->d_errword,

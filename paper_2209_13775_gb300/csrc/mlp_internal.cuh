@@ -36,14 +36,37 @@ struct lcs_mlp {
     float *d_params = nullptr;        // FP32 master copy [MLP_NPARAMS]
     float *d_m = nullptr, *d_v = nullptr;  // Adam moments
     long long adam_steps = 0;
-    unsigned char *d_tiles = nullptr; // inference block (MLP_TILE_BYTES)
-    __nv_bfloat16 *d_wk = nullptr;    // trainer operands: W0 [128][16], W1..W3 [128][128], W4 [16][128]
-    __nv_bfloat16 *d_wt = nullptr;    // transposes: W1^T..W3^T [128][128], W4^T [128][16]
+    unsigned char *d_tiles = nullptr; // operand tiles of inference and training (MLP_TILE_BYTES)
     float *d_grad = nullptr;          // gradient [MLP_NPARAMS]
-    // trainer work space for batches of up to `cap` samples
-    long long cap = 0;
-    void *d_work = nullptr;
+    void *d_work = nullptr;           // trainer's partial gradients
+    double *d_loss = nullptr;         // summed loss of the last lcs_mlp_loss_grad
 };
+
+#ifdef __CUDACC__
+#include "tc_common.cuh"
+
+// parameter i (packed order) of value v into the operand tiles: BF16 weights, FP32 biases
+__device__ __forceinline__ void mlp_store_param(unsigned char *tiles, int i, float v)
+{
+    const auto weight = [&](uint32_t off) { *reinterpret_cast<__nv_bfloat16 *>(tiles + off) = __float2bfloat16_rn(v); };
+    float *bias = reinterpret_cast<float *>(tiles + 106496);
+    if (i < MLP_OFF_B0) {
+        weight(ckm_offset(128, i / 7, i % 7));
+    } else if (i < MLP_OFF_W1) {
+        bias[i - MLP_OFF_B0] = v;
+    } else if (i < MLP_OFF_W4) {
+        const int l = (i - MLP_OFF_W1) / MLP_LAYER_STRIDE, r = (i - MLP_OFF_W1) % MLP_LAYER_STRIDE;
+        if (r < 128 * 128)
+            weight(4096 + 32768u * l + ckm_offset(128, r / 128, r % 128));
+        else
+            bias[128 * (l + 1) + (r - 128 * 128)] = v;
+    } else if (i < MLP_OFF_B4) {
+        weight(102400 + ckm_offset(16, (i - MLP_OFF_W4) / 128, (i - MLP_OFF_W4) % 128));
+    } else {
+        bias[512 + (i - MLP_OFF_B4)] = v;
+    }
+}
+#endif
 
 struct MlpStepArgs {
     const void *tiles;        // inference block in device memory
@@ -94,7 +117,7 @@ lcs_status advect_surrogate(lcs_ctx *ctx, const lcs_field *f, const lcs_seeds *s
                             lcs_flowmap *fm);
 
 // trainer (mlp_train.cu)
-cudaError_t mlp_reserve(lcs_mlp *m, long long B, cudaStream_t s);
+cudaError_t mlp_reserve(lcs_mlp *m, int num_sms);
 cudaError_t mlp_loss_grad(lcs_mlp *m, const float *xyt, long long xstride, const float *disp, long long dstride,
                           long long B, float rho_weight, int num_sms, unsigned *errword, double *d_loss, cudaStream_t s);
 cudaError_t mlp_adam(lcs_mlp *m, const float *grad, double lr, double b1, double b2, double eps, cudaStream_t s);
