@@ -220,6 +220,262 @@ __device__ __forceinline__ double eig_max3(const double *C)
     return (q + p * beta) * is;
 }
 
+// ------------------------------------------------ eigenpairs of 3x3 C, split
+
+// v / 2^ex in double-FP32, from v's bits (no FP64 instructions): zero where below the FP32 range
+__device__ __forceinline__ dfl narrow_scaled(double v, int ex)
+{
+    const int hi = __double2hiint(v);
+    const unsigned lo = (unsigned)__double2loint(v);
+    const int e = ((hi >> 20) & 0x7ff) - 1023 + 127 - ex;   // biased FP32 exponent
+    if (e <= 0 || e >= 255) return {0.0f, 0.0f};
+    const unsigned sg = (unsigned)hi & 0x80000000u;
+    const float h = __uint_as_float(sg | ((unsigned)e << 23) | (((unsigned)hi & 0xfffffu) << 3) | (lo >> 29));
+    const float r = (float)(lo & 0x1fffffffu);              // the bits below: r 2^(e - 127 - 52)
+    const float l = e > 52 ? r * __uint_as_float((unsigned)(e - 52) << 23) : 0.0f;
+    return {h, sg ? -l : l};
+}
+
+__device__ __forceinline__ double widen(dfl a) { return __dadd_rn(widen(a.h), widen(a.l)); }
+
+// 1 / sqrt(a) for a >= 1
+__device__ __forceinline__ dfl df_rsqrt(dfl a)
+{
+    const float y = rsqrtf(a.h);
+    const dfl u = df_mul(a, df_two_prod(y, y));
+    const float e = __fsub_rn(__fsub_rn(1.0f, u.h), u.l);
+    return df_fast_sum(y, __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e), e, __fmul_rn(0.5f, e))));
+}
+
+// tangent of the Jacobi rotation that annihilates apq, d = aqq - app: the smaller root of t^2 + 2 tau t = 1
+__device__ __forceinline__ float jacobi_tan(float d, float apq)
+{
+    const float tau = __fdividef(d, 2.0f * apq);
+    const float t = __fdividef(1.0f, fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
+    return apq == 0.0f ? 0.0f : (fabsf(tau) < 1e18f ? copysignf(t, tau) : __fdividef(0.5f, tau));
+}
+
+// All eigenpairs of the packed 3x3 C by Jacobi rotations whose FP64 work is the part that needs it:
+//  1. four sweeps on C / 2^ex in FP32, the rotations multiplied up as a quaternion (so the matrix V it
+//     stands for is orthonormal to whatever precision V is formed in), which diagonalise C to about 1e-7;
+//  2. V and A = V^T C V in FP64;
+//  3. the rotations left, in double-FP32: their product as R' = R - I and the changes of A's diagonal as
+//     sums of their own, so that both carry 2^-46 of a small quantity.  With t a rotation's tangent and a'
+//     the off-diagonal element it leaves, app' = app - t (apq + a') exactly, whatever the rounding of t;
+//  4. eigenvalues A_kk + changes and vectors V + V R' in FP64.
+// About 185 FP64 operations against 950 for Jacobi rotations in FP64 throughout (eig_jacobi, which serves
+// matrices outside the exponent range here, and 2x2 ones).  Same order and signs as eig_jacobi.
+__device__ __forceinline__ bool eig3_split(const double *C, double *ev, double *Vout)
+{
+    const double dmax = fmax(C[0], fmax(C[3], C[5]));
+    const int ex = ((__double2hiint(dmax) >> 20) & 0x7ff) - 1023;
+    bool fine = dmax > 0.0 && ex > -900 && ex < 900;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) fine = fine && fabs(C[i]) <= 2.0 * dmax;   // false for NaN
+    if (!fine) return false;
+    // 1. FP32
+    float a[3][3], w = 1.0f, q[3] = {0.0f, 0.0f, 0.0f};
+    {
+        const int at[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) a[i][j] = narrow_scaled(C[at[i][j]], ex).h;
+    }
+#pragma unroll 1
+    for (int sweep = 0; sweep < 4; ++sweep) {
+#pragma unroll
+        for (int k = 2; k >= 0; --k) {          // rotation about axis k: planes (0, 1), (0, 2), (1, 2)
+            const int p = k == 0 ? 1 : 0, r = k == 2 ? 1 : 2, o = k;
+            const float apq = a[p][r], t = jacobi_tan(a[r][r] - a[p][p], apq);
+            const float c = rsqrtf(fmaf(t, t, 1.0f)), s = t * c;
+            a[p][p] = fmaf(-t, apq, a[p][p]);
+            a[r][r] = fmaf(t, apq, a[r][r]);
+            a[p][r] = a[r][p] = 0.0f;
+            const float x = a[o][p], y = a[o][r];
+            a[o][p] = a[p][o] = c * x - s * y;
+            a[o][r] = a[r][o] = s * x + c * y;
+            // V <- V J: J[p][r] = s is the rotation by -theta about x and z, by +theta about y; its
+            // quaternion is (1 + c, -+s e_k) up to scale
+            const float jw = 0.5f + 0.5f * c, js = (k == 1 ? 0.5f : -0.5f) * s;
+            const int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
+            const float nw = jw * w - js * q[k], nk = jw * q[k] + js * w;
+            const float n1 = jw * q[k1] + js * q[k2], n2 = jw * q[k2] - js * q[k1];
+            w = nw;
+            q[k] = nk;
+            q[k1] = n1;
+            q[k2] = n2;
+        }
+    }
+    const float nq = rsqrtf(w * w + q[0] * q[0] + q[1] * q[1] + q[2] * q[2]);
+    // 2. V and A in FP64
+    double V[3][3], A[3][3];
+    {
+        const double W = widen(w * nq), X = widen(q[0] * nq), Y = widen(q[1] * nq), Z = widen(q[2] * nq);
+        const double xx = X * X, yy = Y * Y, zz = Z * Z;
+        const double n1 = (W * W - 1.0) + xx + (yy + zz);                  // |q|^2 - 1, of order 1e-7
+        const double s = 2.0 * fma(-n1, fma(-n1, 1.0 - n1, 1.0), 1.0);     // 2 / |q|^2
+        const double sX = s * X, sY = s * Y, sZ = s * Z;
+        const double xy = sX * Y, xz = sX * Z, yz = sY * Z, wx = sX * W, wy = sY * W, wz = sZ * W;
+        V[0][0] = fma(-s, yy + zz, 1.0);
+        V[1][1] = fma(-s, xx + zz, 1.0);
+        V[2][2] = fma(-s, xx + yy, 1.0);
+        V[0][1] = xy - wz;
+        V[1][0] = xy + wz;
+        V[0][2] = xz + wy;
+        V[2][0] = xz - wy;
+        V[1][2] = yz - wx;
+        V[2][1] = yz + wx;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const double w0 = fma(C[0], V[0][j], fma(C[1], V[1][j], C[2] * V[2][j]));
+            const double w1 = fma(C[1], V[0][j], fma(C[3], V[1][j], C[4] * V[2][j]));
+            const double w2 = fma(C[2], V[0][j], fma(C[4], V[1][j], C[5] * V[2][j]));
+#pragma unroll
+            for (int i = 0; i <= j; ++i) A[i][j] = fma(V[0][i], w0, fma(V[1][i], w1, V[2][i] * w2));
+        }
+    }
+    // 3. the rotations left
+    dfl R[3][3], dg[3], d[3], od[3];      // R', diagonal, its changes, off-diagonal opposite axis k
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        dg[i] = narrow_scaled(A[i][i], ex);
+        d[i] = {0.0f, 0.0f};
+#pragma unroll
+        for (int j = 0; j < 3; ++j) R[i][j] = {0.0f, 0.0f};
+    }
+    od[0] = narrow_scaled(A[1][2], ex);
+    od[1] = narrow_scaled(A[0][2], ex);
+    od[2] = narrow_scaled(A[0][1], ex);
+    float widest = 0.0f;
+#pragma unroll 1
+    for (int sweep = 0; sweep < 8; ++sweep) {
+        float most = 0.0f;
+#pragma unroll
+        for (int k = 2; k >= 0; --k) {
+            const int p = k == 0 ? 1 : 0, r = k == 2 ? 1 : 2;
+            const dfl diff = df_add(df_sub(dg[r], dg[p]), df_sub(d[r], d[p]));
+            const float t = jacobi_tan(diff.h, od[k].h);
+            most = fmaxf(most, fabsf(t));
+            const dfl t2 = df_two_prod(t, t), c = df_rsqrt(df_add(t2, 1.0f)), s = df_mul(c, t);
+            const dfl c2 = df_mul(c, c);
+            // c - 1 = -t^2 c^2 / (1 + c), of full relative accuracy
+            const dfl num = df_mul(t2, c2), den = df_add(c, 1.0f);
+            const float q0 = __fdividef(num.h, den.h);
+            const dfl rem = df_sub(num, df_mul(den, q0));
+            const dfl cm1 = df_neg(df_fast_sum(q0, __fdividef(rem.h, den.h)));
+            const dfl left = df_mul(c2, df_sub(df_sub(od[k], df_mul(t2, od[k])), df_mul(diff, t)));
+            const dfl g = df_mul(df_add(od[k], left), t);
+            d[p] = df_sub(d[p], g);
+            d[r] = df_add(d[r], g);
+            od[k] = left;
+            // a[k][p] is the element opposite axis r, a[k][r] the one opposite p
+            const dfl x = od[r], y = od[p];
+            od[r] = df_sub(df_mul(c, x), df_mul(s, y));
+            od[p] = df_add(df_mul(s, x), df_mul(c, y));
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const dfl u = R[i][p], v = R[i][r];
+                dfl nu = df_sub(df_add(u, df_mul(cm1, u)), df_mul(s, v));
+                dfl nv = df_add(df_add(v, df_mul(cm1, v)), df_mul(s, u));
+                if (i == p) {
+                    nu = df_add(nu, cm1);
+                    nv = df_add(nv, s);
+                }
+                if (i == r) {
+                    nu = df_sub(nu, s);
+                    nv = df_add(nv, cm1);
+                }
+                R[i][p] = nu;
+                R[i][r] = nv;
+            }
+        }
+        widest = fmaxf(widest, most);
+        if (most < 0x1p-40f) break;   // what is left is of second order in these
+    }
+    // 4. FP64, in ascending order
+    const double scale = __hiloint2double((1023 + ex) << 20, 0);
+    double e[3], U[3][3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        e[k] = fma(widen(d[k]), scale, A[k][k]);
+        const double r0 = widen(R[0][k]), r1 = widen(R[1][k]), r2 = widen(R[2][k]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) U[k][i] = fma(V[i][0], r0, fma(V[i][1], r1, fma(V[i][2], r2, V[i][k])));
+    }
+    // eigenvalues so near one another that FP32 did not part them leave wide rotations, whose 2^-46 shows in
+    // FP64: one symmetric orthonormalisation, the Rayleigh quotients and the vectors' first-order correction
+    if (widest > 0x1p-12f) {
+        double S[3][3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j <= i; ++j) {
+                S[i][j] = -0.5 * fma(U[i][0], U[j][0], fma(U[i][1], U[j][1], fma(U[i][2], U[j][2], i == j ? -1.0 : 0.0)));
+                S[j][i] = S[i][j];
+            }
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const double u0 = U[0][r], u1 = U[1][r], u2 = U[2][r];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) U[i][r] = fma(S[i][0], u0, fma(S[i][1], u1, fma(S[i][2], u2, U[i][r])));
+        }
+        double w[3][3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            w[k][0] = fma(C[0], U[k][0], fma(C[1], U[k][1], C[2] * U[k][2]));
+            w[k][1] = fma(C[1], U[k][0], fma(C[3], U[k][1], C[4] * U[k][2]));
+            w[k][2] = fma(C[2], U[k][0], fma(C[4], U[k][1], C[5] * U[k][2]));
+            e[k] = fma(U[k][0], w[k][0], fma(U[k][1], w[k][1], U[k][2] * w[k][2]));
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = i + 1; j < 3; ++j) {
+                const double aij = fma(U[i][0], w[j][0], fma(U[i][1], w[j][1], U[i][2] * w[j][2]));
+                const float den = narrow_scaled(e[i] - e[j], ex).h, t = __fdividef(narrow_scaled(aij, ex).h, den);
+                if (den != 0.0f && fabsf(t) < 0x1p-14f) {
+                    const double td = widen(t), cm1 = -0.5 * td * td;   // 1 - cos to t^4
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) {
+                        const double u = U[i][r], v = U[j][r];
+                        U[i][r] = u + fma(td, v, cm1 * u);
+                        U[j][r] = v + fma(-td, u, cm1 * v);
+                    }
+                }
+            }
+    }
+    const auto order = [&](int i, int j) {
+        if (e[j] < e[i]) {
+            double x = e[i];
+            e[i] = e[j];
+            e[j] = x;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                x = U[i][r];
+                U[i][r] = U[j][r];
+                U[j][r] = x;
+            }
+        }
+    };
+    order(0, 1);
+    order(0, 2);
+    order(1, 2);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        double m = U[k][0];
+        if (fabs(U[k][1]) > fabs(m)) m = U[k][1];
+        if (fabs(U[k][2]) > fabs(m)) m = U[k][2];
+        ev[k] = e[k];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) Vout[k * 3 + r] = m < 0.0 ? -U[k][r] : U[k][r];
+    }
+    return true;
+}
+
+// matrices that eig3_split does not take: NaN, zero, extreme exponents
+static __device__ __noinline__ void eig3_jacobi(const double *C, double *ev, double *V) { eig_jacobi<3>(C, ev, V); }
+
 // ------------------------------------------------------- differences and FTLE
 
 // one axis of a seed's differences: mode 1 central (F1 - F2) / 2h, 2 forward (-3 F0 + 4 F1 - F2) / 2h,

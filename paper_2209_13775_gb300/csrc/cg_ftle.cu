@@ -12,7 +12,9 @@
 //    rounded (div_fixed: two operations), so both equal the plain FP64 definition bit for bit.
 //    lambda_max: 2x2 from the quadratic formula; 3x3 from the characteristic cubic of the shifted,
 //    scaled matrix (Smith 1961), whose trigonometric root is taken in FP32 and polished by two FP64
-//    Newton steps, and by Jacobi rotations where the two largest eigenvalues (nearly) coincide;
+//    Newton steps, and by Jacobi rotations where the two largest eigenvalues (nearly) coincide.  The
+//    eigenpairs of a 3x3 C take FP64 for a fifth of their operations (eig3_split): 160^3 seeds 6.23 ->
+//    2.12 ms at three blocks per SM (2.25 ms at two), the FP64 pipe 60% busy;
 //  * the FTLE, an FP32 output: the same formulas in double-FP32 (dfloat_device.cuh), about 200 FP32
 //    operations per seed in 2D and 700 in 3D in place of 65 and 170 FP64 ones, whether or not C or
 //    lambda_max is asked for (one call's FTLE does not depend on its other outputs).  Auxiliary
@@ -96,7 +98,7 @@ __device__ __forceinline__ AxisDiff axis_diff(const CgLaunch &L, const unsigned 
 
 // F64: C, lambda_max or eigenpairs wanted (EIG: the latter), so grad F and C are formed in FP64 as well
 template <int DIM, bool F64, bool EIG, int GM>
-__global__ void __launch_bounds__(256) cg_ftle_kernel(const __grid_constant__ CgLaunch L)
+__global__ void __launch_bounds__(256, EIG ? 3 : 1) cg_ftle_kernel(const __grid_constant__ CgLaunch L)
 {
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int jr = blockIdx.y;        // job relative to job0
@@ -200,7 +202,11 @@ __global__ void __launch_bounds__(256) cg_ftle_kernel(const __grid_constant__ Cg
         }
         if constexpr (EIG) {   // lcs_cg_eigen
             double ev[DIM], V[DIM * DIM];
-            eig_jacobi<DIM>(C, ev, V);
+            if constexpr (DIM == 3) {
+                if (!eig3_split(C, ev, V)) eig3_jacobi(C, ev, V);
+            } else {
+                eig_jacobi<2>(C, ev, V);
+            }
             if (L.eigval) {
 #pragma unroll
                 for (int k = 0; k < DIM; ++k) L.eigval[out * DIM + k] = ev[k];
@@ -283,9 +289,9 @@ cudaError_t launch_cg_ftle(const CgLaunch &L0, cudaStream_t s)
     CgLaunch L = L0;
     cg_prepare(L);
     L.c16 = (uintptr_t)L.C % 16 == 0;
+    const bool eig = L.eigval || L.eigvec;
     const int bt = 256;
     dim3 grid((unsigned)((L.N + bt - 1) / bt), (unsigned)L.njobs);
-    const bool eig = L.eigval || L.eigvec;
     const int gm = L.grad ? GM_VAR : (L.x0aux ? GM_AUX : GM_LATTICE);
     const bool f64 = L.C || L.lam || gm == GM_AUX;
 #define CG_LAUNCH(D, G)                                                   \
