@@ -1,13 +1,14 @@
 // mlp_infer.cu -- the surrogate network on the tcgen05 tensor cores, and the gated
 // surrogate advection built on it.
 //
-// Network (7 -> 128 -> 128 -> 128 -> 128 -> 3, SiLU): per tile of 128 tracers, features
-// phi(x, y, t) are rounded to BF16 into a shared-memory operand tile; each layer is one
-// 128 x N x K MMA chain into a TMEM accumulator (FP32), and its epilogue adds the FP32
-// bias, applies SiLU (h + h tanh(h) with h = z/2, in packed BF16 arithmetic) and writes the
-// BF16 activations back as the next layer's operand.  The weights (104 KB of BF16 operand tiles) and biases stay in
-// shared memory for the whole persistent launch.  Three warpgroups work on three tiles at a
-// time, so each tile's epilogue overlaps the others' MMAs on the tensor core.
+// Network (7 -> 128 -> 128 -> 128 -> 128 -> 3, SiLU).  The features are the rows of every product, as in
+// training: Z_l[out][sample] = W_l H_l, so a thread owns a feature (TMEM lane), its bias is one register
+// and it stores its activations 16 bytes along the samples into the tile [feature][sample] that is the
+// next product's right operand.  Per tile of NS samples the BF16 features phi(x, y, t) are one small
+// operand tile, each layer one MMA chain into an FP32 TMEM accumulator, and its epilogue adds the FP32
+// bias, applies SiLU (h + h tanh(h) with h = z/2, in packed BF16 arithmetic) and overwrites the layer's
+// input tile.  The weights (104 KB of BF16 operand tiles) stay in shared memory for the whole persistent
+// launch.  NG warpgroups work on NG tiles at a time, so a tile's epilogue overlaps the others' MMAs.
 //
 // Gated advection over one surrogate step tau (the audit of each 32-tracer group against
 // the integrator of Eq. 2, and the integrator where the audit fails) runs in two SIMT
@@ -22,11 +23,19 @@
 
 namespace {
 
-constexpr uint32_t OFF_W0 = 0, OFF_W1 = 4096, OFF_W2 = 36864, OFF_W3 = 69632, OFF_W4 = 102400, OFF_BIAS = 106496;
-constexpr uint32_t OFF_WG = MLP_TILE_BYTES;  // per-warpgroup region: phi tile (4 KB) + activations (32 KB)
-constexpr uint32_t WG_BYTES = 4096 + 32768;
-constexpr int NWG = 3;  // warpgroups (tiles in flight) per CTA
-constexpr uint32_t INFER_SMEM = MLP_TILE_BYTES + NWG * WG_BYTES;
+__host__ __device__ constexpr uint32_t w_off(int l) { return l == 0 ? 0u : 4096u + 32768u * (uint32_t)(l - 1); }
+constexpr uint32_t OFF_BIAS = 106496;
+constexpr uint32_t OFF_WG = 108672;    // per-warpgroup regions: activations [128][NS], then phi [16][NS]
+#ifndef MLP_NS
+#define MLP_NS 64
+#endif
+#ifndef MLP_NG
+#define MLP_NG 6
+#endif
+constexpr int NS = MLP_NS, NG = MLP_NG;        // samples per tile, warpgroups (tiles in flight) per CTA
+constexpr uint32_t ACT_BYTES = 128 * NS * 2, WG_BYTES = ACT_BYTES + 16 * NS * 2;
+constexpr uint32_t INFER_SMEM = OFF_WG + NG * WG_BYTES;
+static_assert(INFER_SMEM <= 226 * 1024 && NG * NS <= 512 && NS % 16 == 0, "shared and tensor memory");
 
 __device__ __forceinline__ void wg_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory"); }
 
@@ -50,46 +59,41 @@ __device__ __forceinline__ uint32_t fma_bf16x2(uint32_t a, uint32_t b, uint32_t 
     return d;
 }
 
-// one hidden layer's epilogue for tile row r: the 128 FP32 accumulator columns (all loads in
-// flight before one wait), h = z/2 = acc/2 + b/2 (hb holds b/2) rounded to BF16 pairs, and
-// SiLU(z) = h + h tanh(h) in packed BF16 arithmetic, stored as row r of the next operand tile
-__device__ __forceinline__ void hidden_epilogue(uint32_t ta, const float *hb, unsigned char *tile, int r)
+// one hidden layer's epilogue for feature f of a tile: h = z/2 = acc/2 + b/2 (hb = b/2) rounded to BF16
+// pairs, SiLU(z) = h + h tanh(h) in packed BF16 arithmetic, stored as row f of the next operand tile
+__device__ __forceinline__ void hidden_epilogue(uint32_t ta, float hb, unsigned char *tile, int f)
 {
+    const float2 half = make_float2(0.5f, 0.5f), b2 = make_float2(hb, hb);
 #pragma unroll
-    for (int half = 0; half < 128; half += 64) {
-        uint32_t acc[64];
-        tmem_ld32_async(ta + half, acc);
-        tmem_ld32_async(ta + half + 32, acc + 32);
-        tmem_wait_ld32(acc);
-        tmem_wait_ld32(acc + 32);
+    for (int c0 = 0; c0 < NS; c0 += 16) {
+        float acc[16];
+        tmem_ld16(ta + c0, acc);
 #pragma unroll
-        for (int c = 0; c < 64; c += 8) {
+        for (int c = 0; c < 16; c += 8) {
             uint32_t w[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const float h0 = fmaf(__uint_as_float(acc[c + 2 * j]), 0.5f, hb[half + c + 2 * j]);
-                const float h1 = fmaf(__uint_as_float(acc[c + 2 * j + 1]), 0.5f, hb[half + c + 2 * j + 1]);
-                const uint32_t h2 = pack_bf16(h0, h1);
+                const float2 h = __ffma2_rn(make_float2(acc[c + 2 * j], acc[c + 2 * j + 1]), half, b2);
+                const uint32_t h2 = pack_bf16(h.x, h.y);
                 w[j] = fma_bf16x2(h2, tanh_bf16x2(h2), h2);
             }
-            *reinterpret_cast<uint4 *>(tile + ckm_offset(128, r, half + c)) = make_uint4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<uint4 *>(tile + ckm_offset(128, f, c0 + c)) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
 }
 
-__global__ void __launch_bounds__(NWG * 128, 1) mlp_step_kernel(MlpStepArgs A)
+__global__ void __launch_bounds__(NG * 128, 1) mlp_step_kernel(const MlpStepArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint64_t bar_w, bar_g[NWG];
+    __shared__ uint64_t bar_w, bar_g[NG];
     __shared__ uint32_t tmem_base;
-    __shared__ int abort_flag[NWG];
+    __shared__ int abort_flag[NG];
     const int tid = threadIdx.x, warp = tid >> 5;
     const int g = warp >> 2;           // warpgroup
-    const int r = tid & 127;           // tile row = TMEM lane
-    const int wq = warp & 3;
+    const int f = tid & 127;           // feature = TMEM lane
     if (tid == 0) {
         mbar_init(&bar_w, 1);
-        for (int q = 0; q < NWG; ++q) {
+        for (int q = 0; q < NG; ++q) {
             mbar_init(&bar_g[q], 1);
             abort_flag[q] = 0;
         }
@@ -104,56 +108,59 @@ __global__ void __launch_bounds__(NWG * 128, 1) mlp_step_kernel(MlpStepArgs A)
         bulk_g2s(smem, A.tiles, MLP_TILE_BYTES, &bar_w);
     }
     const bool have_w = !__syncthreads_or(!tc_wait(&bar_w, 0, A.errword));
-    if (have_w) {  // hidden-layer biases are used halved (the epilogue works with z / 2)
-        float *b = reinterpret_cast<float *>(smem + OFF_BIAS);
-        for (int q = tid; q < 512; q += blockDim.x) b[q] *= 0.5f;
-        __syncthreads();
-    }
-    const uint32_t tmem = tmem_base + (uint32_t)(g * 128);
-    unsigned char *sPhi = smem + OFF_WG + g * WG_BYTES;
-    unsigned char *sAct = sPhi + 4096;
+    const uint32_t tmem = tmem_base + (uint32_t)(g * NS);
+    unsigned char *sAct = smem + OFF_WG + g * WG_BYTES;
+    unsigned char *sPhi = sAct + ACT_BYTES;
+    float *sOut = reinterpret_cast<float *>(sPhi);     // [3][NS] outputs (phi is done by then)
     const float *bias = reinterpret_cast<const float *>(smem + OFF_BIAS);
     const uint32_t uPhi = smem_u32(sPhi), uAct = smem_u32(sAct), uW = smem_u32(smem);
-    const uint32_t id128 = tc_idesc_bf16(128, 128), id16 = tc_idesc_bf16(128, 16);
-    const long long ntiles = (A.n + 127) / 128;
+    // A (weights) with K leading, B (activations, features) with the samples leading: descriptor bit 16
+    const uint32_t idesc = tc_idesc_bf16(128, NS) | (1u << 16);
+    float hb[4] = {0.0f, 0.0f, 0.0f, 0.0f};            // hidden-layer biases, halved
+    if (have_w)
+#pragma unroll
+        for (int l = 0; l < 4; ++l) hb[l] = 0.5f * bias[l * 128 + f];
+    const long long ntiles = (A.n + NS - 1) / NS;
     unsigned phase = 0;
-    for (long long tile = (long long)blockIdx.x * NWG + g; have_w && tile < ntiles; tile += (long long)NWG * gridDim.x) {
-        const long long i = tile * 128 + r;
-        const bool live = i < A.n;
+    for (long long tile = blockIdx.x + (long long)gridDim.x * g; have_w && tile < ntiles;
+         tile += (long long)NG * gridDim.x) {
+        const long long i = tile * NS + f;
+        const bool live = f < NS && i < A.n;
         float x = 0.0f, y = 0.0f, t = A.t_uniform;
         if (live) {
             x = A.x[i];
             y = A.x[A.stride + i];
             if (A.t) t = A.t[i];
         }
-        {   // features -> BF16 row r of the phi tile (K = 16, columns 7..15 zero)
-            float sw, cw, sx, cx, sy, cy;
-            sincosf(A.omega * t, &sw, &cw);
-            sincosf(A.kx * x, &sx, &cx);
-            sincosf(A.ky * y, &sy, &cy);
-            const uint4 lo = make_uint4(pack_bf16(x - A.cx, y - A.cy), pack_bf16(sw, cw), pack_bf16(sx, cx),
-                                        pack_bf16(sy, 0.0f));
-            *reinterpret_cast<uint4 *>(sPhi + ckm_offset(128, r, 0)) = lo;
-            *reinterpret_cast<uint4 *>(sPhi + ckm_offset(128, r, 8)) = make_uint4(0, 0, 0, 0);
+        if (f < NS) {   // features -> BF16 column f of the phi tile (K = 16, rows 7..15 zero)
+            float v[8];
+            float cy;
+            sincosf(A.omega * t, &v[2], &v[3]);
+            sincosf(A.kx * x, &v[4], &v[5]);
+            sincosf(A.ky * y, &v[6], &cy);
+            v[0] = x - A.cx;
+            v[1] = y - A.cy;
+            v[7] = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                *reinterpret_cast<__nv_bfloat16 *>(sPhi + ckm_offset(16, k, f)) = __float2bfloat16_rn(k < 7 ? v[k & 7] : 0.0f);
         }
-        float o[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
         for (int l = 0; l < 5; ++l) {
             fence_async_smem();
             tc_fence_before();
             wg_sync(g);
-            if (r == 0) {
+            if (f == 0) {
                 tc_fence_after();
                 if (l == 0) {
-                    tc_mma(tmem, tc_desc(uPhi, 2048, 128), tc_desc(uW + OFF_W0, 2048, 128), id128, false);
+                    tc_mma(tmem, tc_desc(uW, 2048, 128), tc_desc(uPhi, 128, 256), idesc, false);
                 } else {
-                    const uint32_t wofs = l == 1 ? OFF_W1 : l == 2 ? OFF_W2 : l == 3 ? OFF_W3 : OFF_W4;
+                    // W4 has 16 rows: the product's rows from 16 on read what follows it and are not used
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {
-                        const uint64_t ad = tc_desc(uAct + kk * 4096, 2048, 128);
-                        const uint64_t bd = l < 4 ? tc_desc(uW + wofs + kk * 4096, 2048, 128)
-                                                  : tc_desc(uW + wofs + kk * 512, 256, 128);
-                        tc_mma(tmem, ad, bd, l < 4 ? id128 : id16, kk > 0);
-                    }
+                    for (int kk = 0; kk < 8; ++kk)
+                        tc_mma(tmem, l < 4 ? tc_desc(uW + w_off(l) + kk * 4096, 2048, 128)
+                                           : tc_desc(uW + w_off(4) + kk * 512, 256, 128),
+                               tc_desc(uAct + kk * 256, 128, 2048), idesc, kk > 0);
                 }
                 tc_commit(&bar_g[g]);
             }
@@ -162,18 +169,26 @@ __global__ void __launch_bounds__(NWG * 128, 1) mlp_step_kernel(MlpStepArgs A)
             wg_sync(g);  // every thread of the warpgroup sees the same abort flag
             if (abort_flag[g]) break;
             tc_fence_after();
-            const uint32_t ta = tmem + ((uint32_t)(wq * 32) << 16);
+            const uint32_t ta = tmem + ((uint32_t)((warp & 3) * 32) << 16);
             if (l < 4) {
-                hidden_epilogue(ta, bias + l * 128, sAct, r);
-            } else {
-                float v[16];
-                tmem_ld16(ta, v);
-                o[0] = v[0] + bias[512];
-                o[1] = v[1] + bias[513];
-                o[2] = v[2] + bias[514];
+                hidden_epilogue(ta, hb[l], sAct, f);
+            } else if ((warp & 3) == 0) {
+                const float bo = f < 3 ? bias[512 + f] : 0.0f;
+#pragma unroll
+                for (int c = 0; c < NS; c += 16) {
+                    float v[16];
+                    tmem_ld16(ta + c, v);
+                    if (f < 3)
+#pragma unroll
+                        for (int j = 0; j < 16; j += 4)
+                            *reinterpret_cast<float4 *>(sOut + f * NS + c + j) =
+                                make_float4(v[j] + bo, v[j + 1] + bo, v[j + 2] + bo, v[j + 3] + bo);
+                }
             }
         }
         if (abort_flag[g]) break;
+        wg_sync(g);
+        const float o[3] = {sOut[f % NS], sOut[NS + f % NS], sOut[2 * NS + f % NS]};
         if (live) {
             if (A.mode == 0) {
                 A.out0[i] = o[0];
@@ -185,6 +200,7 @@ __global__ void __launch_bounds__(NWG * 128, 1) mlp_step_kernel(MlpStepArgs A)
                 A.out2[i] = o[2];
             }
         }
+        wg_sync(g);   // the outputs are read before the next tile's features take their place
     }
     tc_fence_before();
     __syncthreads();
@@ -299,9 +315,9 @@ cudaError_t launch_mlp_step(const MlpStepArgs &A, int num_sms, cudaStream_t s)
     if (A.n <= 0) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(mlp_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)INFER_SMEM);
     if (e != cudaSuccess) return e;
-    const long long pairs = ((A.n + 127) / 128 + NWG - 1) / NWG;
-    const int grid = (int)(pairs < num_sms ? pairs : num_sms);
-    mlp_step_kernel<<<grid, NWG * 128, INFER_SMEM, s>>>(A);
+    const long long tiles = (A.n + NS - 1) / NS;
+    const int grid = (int)(tiles < num_sms ? tiles : num_sms);
+    mlp_step_kernel<<<grid, NG * 128, INFER_SMEM, s>>>(A);
     return cudaGetLastError();
 }
 
