@@ -9,6 +9,10 @@
 // bias, applies SiLU (h + h tanh(h) with h = z/2, in packed BF16 arithmetic) and overwrites the layer's
 // input tile.  The weights (104 KB of BF16 operand tiles) stay in shared memory for the whole persistent
 // launch.  NG warpgroups work on NG tiles at a time, so a tile's epilogue overlaps the others' MMAs.
+// The MUFU bounds it (two slots per tanh of a BF16 pair: 73% of its cycles, 0.23 ms at full rate for
+// 2,097,229 evaluations): 0.450 ms with the samples as rows and three tiles of 128 per SM, 0.330 with the
+// features as rows and six tiles of 64, 0.322 with weights in tensor memory and points loaded ahead (657
+// TFLOP/s).  48 x 8: 0.344; 96 x 4: 0.343; 128 x 3: 0.364; 64 x 5: 0.369.
 //
 // Gated advection over one surrogate step tau (the audit of each 32-tracer group against
 // the integrator of Eq. 2, and the integrator where the audit fails) runs in two SIMT
@@ -26,16 +30,12 @@ namespace {
 __host__ __device__ constexpr uint32_t w_off(int l) { return l == 0 ? 0u : 4096u + 32768u * (uint32_t)(l - 1); }
 constexpr uint32_t OFF_BIAS = 106496;
 constexpr uint32_t OFF_WG = 108672;    // per-warpgroup regions: activations [128][NS], then phi [16][NS]
-#ifndef MLP_NS
-#define MLP_NS 64
-#endif
-#ifndef MLP_NG
-#define MLP_NG 6
-#endif
-constexpr int NS = MLP_NS, NG = MLP_NG;        // samples per tile, warpgroups (tiles in flight) per CTA
+constexpr int NS = 64, NG = 6;         // samples per tile, warpgroups (tiles in flight) per CTA
+constexpr int TW = 2;                  // hidden layers whose weights the products take from tensor memory
+constexpr uint32_t TM_ACC = 64 * TW;   // TMEM: W1..W_TW (64 columns each), then an accumulator per warpgroup
 constexpr uint32_t ACT_BYTES = 128 * NS * 2, WG_BYTES = ACT_BYTES + 16 * NS * 2;
 constexpr uint32_t INFER_SMEM = OFF_WG + NG * WG_BYTES;
-static_assert(INFER_SMEM <= 226 * 1024 && NG * NS <= 512 && NS % 16 == 0, "shared and tensor memory");
+static_assert(INFER_SMEM <= 226 * 1024 && TM_ACC + NG * NS <= 512 && NS % 16 == 0, "shared and tensor memory");
 
 __device__ __forceinline__ void wg_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory"); }
 
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(NG * 128, 1) mlp_step_kernel(const MlpStepArgs
         bulk_g2s(smem, A.tiles, MLP_TILE_BYTES, &bar_w);
     }
     const bool have_w = !__syncthreads_or(!tc_wait(&bar_w, 0, A.errword));
-    const uint32_t tmem = tmem_base + (uint32_t)(g * NS);
+    const uint32_t tmem = tmem_base + TM_ACC + (uint32_t)(g * NS);
     unsigned char *sAct = smem + OFF_WG + g * WG_BYTES;
     unsigned char *sPhi = sAct + ACT_BYTES;
     float *sOut = reinterpret_cast<float *>(sPhi);     // [3][NS] outputs (phi is done by then)
@@ -120,18 +120,43 @@ __global__ void __launch_bounds__(NG * 128, 1) mlp_step_kernel(const MlpStepArgs
     if (have_w)
 #pragma unroll
         for (int l = 0; l < 4; ++l) hb[l] = 0.5f * bias[l * 128 + f];
+    // W1 and W2 into tensor memory, where the products take them from: read from shared memory by every MMA
+    // they are 4 KB of its 6 KB (0.328 ms with all of them there, 0.325 with W1 moved, 0.322 with both; a
+    // third leaves room for five accumulators only: 0.347)
+    if (have_w && g < TW) {
+        const uint32_t tw = tmem_base + 64 * g + ((uint32_t)((warp & 3) * 32) << 16);
+#pragma unroll
+        for (int c = 0; c < 64; c += 16) {
+            uint32_t r[16];
+#pragma unroll
+            for (int q = 0; q < 16; q += 4)
+                *reinterpret_cast<uint4 *>(r + q) =
+                    *reinterpret_cast<const uint4 *>(smem + w_off(1 + g) + ckm_offset(128, f, 2 * (c + q)));
+            tmem_st16(tw + c, r);
+        }
+        tmem_wait_st();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
     const long long ntiles = (A.n + NS - 1) / NS;
     unsigned phase = 0;
+    // a tile's points are loaded while the tile before it goes through the network
+    float px = 0.0f, py = 0.0f, pt = A.t_uniform;
+    const auto load = [&](long long tile) {
+        const long long i = tile * NS + f;
+        if (f < NS && i < A.n) {
+            px = A.x[i];
+            py = A.x[A.stride + i];
+            if (A.t) pt = A.t[i];
+        }
+    };
+    load(blockIdx.x + (long long)gridDim.x * g);
     for (long long tile = blockIdx.x + (long long)gridDim.x * g; have_w && tile < ntiles;
          tile += (long long)NG * gridDim.x) {
         const long long i = tile * NS + f;
         const bool live = f < NS && i < A.n;
-        float x = 0.0f, y = 0.0f, t = A.t_uniform;
-        if (live) {
-            x = A.x[i];
-            y = A.x[A.stride + i];
-            if (A.t) t = A.t[i];
-        }
+        const float x = px, y = py, t = pt;
         if (f < NS) {   // features -> BF16 column f of the phi tile (K = 16, rows 7..15 zero)
             float v[8];
             float cy;
@@ -145,6 +170,7 @@ __global__ void __launch_bounds__(NG * 128, 1) mlp_step_kernel(const MlpStepArgs
             for (int k = 0; k < 16; ++k)
                 *reinterpret_cast<__nv_bfloat16 *>(sPhi + ckm_offset(16, k, f)) = __float2bfloat16_rn(k < 7 ? v[k & 7] : 0.0f);
         }
+        load(tile + (long long)NG * gridDim.x);
 #pragma unroll
         for (int l = 0; l < 5; ++l) {
             fence_async_smem();
@@ -158,9 +184,13 @@ __global__ void __launch_bounds__(NG * 128, 1) mlp_step_kernel(const MlpStepArgs
                     // W4 has 16 rows: the product's rows from 16 on read what follows it and are not used
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)
-                        tc_mma(tmem, l < 4 ? tc_desc(uW + w_off(l) + kk * 4096, 2048, 128)
-                                           : tc_desc(uW + w_off(4) + kk * 512, 256, 128),
-                               tc_desc(uAct + kk * 256, 128, 2048), idesc, kk > 0);
+                        if (l <= TW)
+                            tc_mma_ts(tmem, tmem_base + 64 * (l - 1) + 8 * kk, tc_desc(uAct + kk * 256, 128, 2048),
+                                      idesc, kk > 0);
+                        else
+                            tc_mma(tmem, l < 4 ? tc_desc(uW + w_off(l) + kk * 4096, 2048, 128)
+                                               : tc_desc(uW + w_off(4) + kk * 512, 256, 128),
+                                   tc_desc(uAct + kk * 256, 128, 2048), idesc, kk > 0);
                 }
                 tc_commit(&bar_g[g]);
             }
