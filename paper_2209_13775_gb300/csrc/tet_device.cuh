@@ -260,6 +260,132 @@ __device__ __forceinline__ void tet_interp_grad(const TetDev &T, int c, const fl
     u[2] = acc[2];
 }
 
+// A tracer's register cache on tets, as TriCache on triangles: the map of the cell its last walk ended in and
+// the vertex velocities, as stored, of the cell and frame interval it last interpolated.  Fixed RK4 steps
+// are short against cells and frame gaps, so most stage points find both; a hit uses exactly what a reload
+// would read, so the results are the same bits.
+template <int ST>
+struct TetCache {
+    float4 r0, r1, r2;
+    int mc;          // cell of r0..r2 (-1: none)
+    int pc, pk;      // cell and interval of the vertex words (-1: none)
+    static constexpr int WORDS = ST == LCS_F32 ? 8 : 4;
+    unsigned w[4][WORDS];
+};
+
+template <int ST>
+__device__ __forceinline__ void tet_cache_init(TetCache<ST> &cc)
+{
+    cc.mc = cc.pc = cc.pk = -1;
+}
+
+// tet_locate with the map of each visited cell taken from, or put into, the cache
+template <int ST>
+__device__ __forceinline__ int tet_locate_cached(const TetDev &T, const float *x, int *cell, float *lam, TetCache<ST> &cc)
+{
+    int c = *cell;
+    if ((unsigned)c >= (unsigned)T.ncells) c = 0;
+    for (int it = 0; it < T.walk_limit; ++it) {
+        const float4 *rec = T.tmap + 4 * (size_t)c;
+        if (c != cc.mc) {
+            asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                : "=f"(cc.r0.x), "=f"(cc.r0.y), "=f"(cc.r0.z), "=f"(cc.r0.w), "=f"(cc.r1.x), "=f"(cc.r1.y), "=f"(cc.r1.z),
+                  "=f"(cc.r1.w)
+                : "l"(rec));
+            cc.r2 = __ldg(rec + 2);
+            cc.mc = c;
+        }
+        tet_bary_rows(cc.r0, cc.r1, cc.r2, x, lam);
+        const float lm = fminf(fminf(lam[0], lam[1]), fminf(lam[2], lam[3]));
+        if (lm >= -T.tol) {
+            *cell = c;
+            return TET_INSIDE;
+        }
+        // the face of the first smallest coordinate
+        int jm = 0;
+        float lo = lam[0];
+#pragma unroll
+        for (int j = 1; j < 4; ++j)
+            if (lam[j] < lo) {
+                lo = lam[j];
+                jm = j;
+            }
+        const int n = __ldg(reinterpret_cast<const int *>(rec + 3) + jm);
+        if (n < 0) {
+            *cell = c;
+            return T.convex ? TET_OUTSIDE : tet_bin_scan(T, x, cell, lam);
+        }
+        c = n;
+    }
+    *cell = c;
+    return TET_WALKFAIL;
+}
+
+template <int ST>
+__device__ __forceinline__ void tet_words(const char *fp, int v, unsigned *w)
+{
+    if constexpr (ST == LCS_F32) {
+        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+            : "l"(fp + 32 * (size_t)v));
+    } else {
+        const uint4 r = __ldg(reinterpret_cast<const uint4 *>(fp) + v);
+        w[0] = r.x;
+        w[1] = r.y;
+        w[2] = r.z;
+        w[3] = r.w;
+    }
+}
+
+// the two frames' velocities in a vertex's words (u_k, 0, u_{k+1}, 0)
+template <int ST>
+__device__ __forceinline__ void tet_unpack(const unsigned *w, float *ua, float *ub)
+{
+    if constexpr (ST == LCS_F32) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            ua[q] = __uint_as_float(w[q]);
+            ub[q] = __uint_as_float(w[4 + q]);
+        }
+    } else {
+        const float2 a = ST == LCS_F16 ? tet_h2f(w[0]) : tet_b2f(w[0]), b = ST == LCS_F16 ? tet_h2f(w[1]) : tet_b2f(w[1]);
+        const float2 c = ST == LCS_F16 ? tet_h2f(w[2]) : tet_b2f(w[2]), d = ST == LCS_F16 ? tet_h2f(w[3]) : tet_b2f(w[3]);
+        ua[0] = a.x;
+        ua[1] = a.y;
+        ua[2] = b.x;
+        ub[0] = c.x;
+        ub[1] = c.y;
+        ub[2] = d.x;
+    }
+}
+
+// tet_interp in interval k (pairs at fp) with the vertex words taken from, or put into, the cache
+template <int ST>
+__device__ __forceinline__ void tet_interp_cached(const TetDev &T, int c, int k, const float *lam, const char *fp, float a,
+                                                  float *u, TetCache<ST> &cc)
+{
+    if (c != cc.pc || k != cc.pk) {
+        const int4 t = __ldg(T.tets + c);
+        tet_words<ST>(fp, t.x, cc.w[0]);
+        tet_words<ST>(fp, t.y, cc.w[1]);
+        tet_words<ST>(fp, t.z, cc.w[2]);
+        tet_words<ST>(fp, t.w, cc.w[3]);
+        cc.pc = c;
+        cc.pk = k;
+    }
+    const float g = 1.0f - a;
+    float acc[3] = {0.0f, 0.0f, 0.0f}, va[3], vb[3];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        tet_unpack<ST>(cc.w[i], va, vb);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) acc[q] = fmaf(lam[i], a == 0.0f ? va[q] : fmaf(a, vb[q], g * va[q]), acc[q]);
+    }
+    u[0] = acc[0];
+    u[1] = acc[1];
+    u[2] = acc[2];
+}
+
 // ------------------------------------------------------------ exact orientation
 
 // error-free transformations (Knuth's TwoSum; the FMA residual of a product)
