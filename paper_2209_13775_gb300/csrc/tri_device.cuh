@@ -108,7 +108,7 @@ struct TriCache {
     float2 v;
     int mc;        // cell of m, v (-1: none)
     int pc, pk;    // cell and interval of ua, ub (-1: none)
-    float ua[3][2], ub[3][2];
+    float2 ua[3], ub[3];
 };
 
 __device__ __forceinline__ void tri_cache_init(TriCache &cc)
@@ -186,57 +186,46 @@ struct TriPair;
 
 template <>
 struct TriPair<LCS_F32> {
-    static __device__ __forceinline__ void ld(const char *f, int v, float *ua, float *ub)
+    static __device__ __forceinline__ void ld(const char *f, int v, float2 &ua, float2 &ub)
     {
         const float4 r = __ldg(reinterpret_cast<const float4 *>(f) + v);
-        ua[0] = r.x;
-        ua[1] = r.y;
-        ub[0] = r.z;
-        ub[1] = r.w;
+        ua = make_float2(r.x, r.y);
+        ub = make_float2(r.z, r.w);
     }
 };
 
 template <>
 struct TriPair<LCS_F16> {
-    static __device__ __forceinline__ void ld(const char *f, int v, float *ua, float *ub)
+    static __device__ __forceinline__ void ld(const char *f, int v, float2 &ua, float2 &ub)
     {
         const uint2 r = __ldg(reinterpret_cast<const uint2 *>(f) + v);
-        const float2 a = tet_h2f(r.x), b = tet_h2f(r.y);
-        ua[0] = a.x;
-        ua[1] = a.y;
-        ub[0] = b.x;
-        ub[1] = b.y;
+        ua = tet_h2f(r.x);
+        ub = tet_h2f(r.y);
     }
 };
 
 template <>
 struct TriPair<LCS_BF16> {
-    static __device__ __forceinline__ void ld(const char *f, int v, float *ua, float *ub)
+    static __device__ __forceinline__ void ld(const char *f, int v, float2 &ua, float2 &ub)
     {
         const uint2 r = __ldg(reinterpret_cast<const uint2 *>(f) + v);
-        const float2 a = tet_b2f(r.x), b = tet_b2f(r.y);
-        ua[0] = a.x;
-        ua[1] = a.y;
-        ub[0] = b.x;
-        ub[1] = b.y;
+        ua = tet_b2f(r.x);
+        ub = tet_b2f(r.y);
     }
 };
 
 // u = sum_i lam_i [(1 - a) u_k + a u_{k+1}](vertex i) from the vertices' pairs (u_k, u_{k+1}).
 // Every pair holds finite values (a single frame is paired with itself), so a = 0 gives u_k
 // exactly without a select: 0 * u_{k+1} + 1 * u_k.
-__device__ __forceinline__ void tri_blend(const float *lam, const float (*ua)[2], const float (*ub)[2], float a,
-                                          float *u)
+// Both components go through the two-lane FP32 instructions.
+__device__ __forceinline__ float2 tri_blend(const float *lam, const float2 *ua, const float2 *ub, float a)
 {
-    const float g = 1.0f - a;
-    float acc[2] = {0.0f, 0.0f};
+    const float2 a2 = make_float2(a, a), g2 = make_float2(1.0f - a, 1.0f - a);
+    float2 acc = make_float2(0.0f, 0.0f);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-            acc[q] = fmaf(lam[i], fmaf(a, ub[i][q], g * ua[i][q]), acc[q]);
-    u[0] = acc[0];
-    u[1] = acc[1];
+        acc = __ffma2_rn(make_float2(lam[i], lam[i]), __ffma2_rn(a2, ub[i], __fmul2_rn(g2, ua[i])), acc);
+    return acc;
 }
 
 // tri_blend of cell c's vertices from the interval pair at fp
@@ -244,17 +233,19 @@ template <int ST>
 __device__ __forceinline__ void tri_interp(const TriDev &T, int c, const float *lam, const char *fp, float a, float *u)
 {
     const int4 t = __ldg(T.tris + c);
-    float ua[3][2], ub[3][2];
+    float2 ua[3], ub[3];
     TriPair<ST>::ld(fp, t.x, ua[0], ub[0]);
     TriPair<ST>::ld(fp, t.y, ua[1], ub[1]);
     TriPair<ST>::ld(fp, t.z, ua[2], ub[2]);
-    tri_blend(lam, ua, ub, a, u);
+    const float2 r = tri_blend(lam, ua, ub, a);
+    u[0] = r.x;
+    u[1] = r.y;
 }
 
 // tri_interp in interval k (pairs at fp) with the vertex pairs taken from, or put into, the cache
 template <int ST>
-__device__ __forceinline__ void tri_interp_cached(const TriDev &T, int c, int k, const float *lam, const char *fp,
-                                                  float a, float *u, TriCache &cc)
+__device__ __forceinline__ float2 tri_interp_cached(const TriDev &T, int c, int k, const float *lam, const char *fp,
+                                                    float a, TriCache &cc)
 {
     if (c != cc.pc || k != cc.pk) {
         const int4 t = __ldg(T.tris + c);
@@ -264,7 +255,7 @@ __device__ __forceinline__ void tri_interp_cached(const TriDev &T, int c, int k,
         cc.pc = c;
         cc.pk = k;
     }
-    tri_blend(lam, cc.ua, cc.ub, a, u);
+    return tri_blend(lam, cc.ua, cc.ub, a);
 }
 
 // tri_interp's u plus the Jacobian of the P1 interpolant, constant in the triangle, with c's map m
@@ -276,7 +267,7 @@ __device__ __forceinline__ void tri_interp_grad(const TriDev &T, int c, const fl
                                                 const char *fp, float a, float *u, float (*J)[2])
 {
     const int4 t = __ldg(T.tris + c);
-    float ua[3][2], ub[3][2];
+    float2 ua[3], ub[3];
     TriPair<ST>::ld(fp, t.x, ua[0], ub[0]);
     TriPair<ST>::ld(fp, t.y, ua[1], ub[1]);
     TriPair<ST>::ld(fp, t.z, ua[2], ub[2]);
@@ -291,7 +282,8 @@ __device__ __forceinline__ void tri_interp_grad(const TriDev &T, int c, const fl
     for (int i = 0; i < 3; ++i) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            const float v = fmaf(a, ub[i][q], g * ua[i][q]);
+            const float va = q == 0 ? ua[i].x : ua[i].y, vb = q == 0 ? ub[i].x : ub[i].y;
+            const float v = fmaf(a, vb, g * va);
             acc[q] = fmaf(lam[i], v, acc[q]);
 #pragma unroll
             for (int d = 0; d < 2; ++d) J[q][d] = fmaf(gr[i][d], v, J[q][d]);
