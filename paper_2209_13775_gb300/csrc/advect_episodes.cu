@@ -414,32 +414,84 @@ __device__ __forceinline__ int axis_cell_ext(const RectParams &P, const SliceGeo
     }
 }
 
-// Trilinear weights of x (make_stencil's products) and the extended base node of its cell.
+// Extended cell e and fraction f of x on every axis, as axis_cell_ext gives them.  PM >= 0 (boxes whose axes
+// all wrap, or all end, of at most FLOOR_MAX_NODES nodes): the floor without the conversion pipe, x and y in
+// two-lane FP32 instructions; an index that is out of range, which includes every coordinate beyond the reach
+// of that floor, goes back to axis_cell_ext's floor and wraps.
 template <int PM>
-__device__ __forceinline__ int stencil_ext(const RectParams &P, const SliceGeom &G, const float *x, float *w)
+__device__ __forceinline__ void cell_ext(const RectParams &P, const SliceGeom &G, const float *x, int *e, float *f)
 {
-    float fx, fy, fz;
-    int rx, ry, rz;
-    bool out = false;
-    int ix = axis_cell_ext<PM>(P, G, 0, x[0], fx, rx, out);
-    int iy = axis_cell_ext<PM>(P, G, 1, x[1], fy, ry, out);
-    int iz = axis_cell_ext<PM>(P, G, 2, x[2], fz, rz, out);
-    if (out) {   // rare: wrap every periodic axis into the box (the others are already in range)
-        if (per_axis<PM>(P, 0)) ix = wrap_index_slow(rx, P.n[0]) + G.H[0];
-        if (per_axis<PM>(P, 1)) iy = wrap_index_slow(ry, P.n[1]) + G.H[1];
-        if (per_axis<PM>(P, 2)) iz = wrap_index_slow(rz, P.n[2]) + G.H[2];
+    if constexpr (PM >= 0) {
+        const float2 M2 = make_float2(FLOOR_MAGIC, FLOOR_MAGIC), m1 = make_float2(-1.0f, -1.0f);
+        const float2 no = make_float2(-P.origin[0], -P.origin[1]), ih = make_float2(P.inv_h[0], P.inv_h[1]);
+        float2 q = make_float2(x[0], x[1]);
+        float z = x[2];
+        if constexpr (PM == 0) {
+            q.x = fminf(fmaxf(q.x, P.origin[0]), P.hi_node[0]);
+            q.y = fminf(fmaxf(q.y, P.origin[1]), P.hi_node[1]);
+            z = fminf(fmaxf(z, P.origin[2]), P.hi_node[2]);
+        }
+        const float2 s = __fmul2_rn(__fadd2_rn(q, no), ih);
+        const float sz = __fmul_rn(z - P.origin[2], P.inv_h[2]);
+        float2 t = __fadd2_rd(s, M2);
+        float tz = __fadd_rd(sz, FLOOR_MAGIC);
+        if constexpr (PM == 0) {
+            t.x = fminf(t.x, FLOOR_MAGIC + (float)(P.n[0] - 2));
+            t.y = fminf(t.y, FLOOR_MAGIC + (float)(P.n[1] - 2));
+            tz = fminf(tz, FLOOR_MAGIC + (float)(P.n[2] - 2));
+        }
+        const float2 fr = __fadd2_rn(s, __ffma2_rn(t, m1, M2));
+        f[0] = fr.x;
+        f[1] = fr.y;
+        f[2] = __fsub_rn(sz, tz - FLOOR_MAGIC);
+        constexpr int H = PM == 0 ? 0 : SLICE_HALO;
+        e[0] = floor_index(t.x) + H;
+        e[1] = floor_index(t.y) + H;
+        e[2] = floor_index(tz) + H;
+        if constexpr (PM == 7) {
+            if ((unsigned)e[0] > (unsigned)(G.N[0] - 2) || (unsigned)e[1] > (unsigned)(G.N[1] - 2) ||
+                (unsigned)e[2] > (unsigned)(G.N[2] - 2)) {   // rare
+                const float sd[3] = {s.x, s.y, sz};
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const float fl = floorf(sd[d]);
+                    f[d] = sd[d] - fl;
+                    const int raw = (int)fl, g = raw + H;
+                    e[d] = (unsigned)g > (unsigned)(G.N[d] - 2) ? wrap_index_slow(raw, P.n[d]) + H : g;
+                }
+            }
+        }
+    } else {
+        int r[3];
+        bool out = false;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) e[d] = axis_cell_ext<PM>(P, G, d, x[d], f[d], r[d], out);
+        if (out) {   // rare: wrap every periodic axis into the box (the others are already in range)
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                if (per_axis<PM>(P, d)) e[d] = wrap_index_slow(r[d], P.n[d]) + G.H[d];
+        }
     }
-    const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
-    const float a = gy * gz, b = fy * gz, c = gy * fz, d = fy * fz;
+}
+
+// Trilinear weights of x (make_stencil's products), its fractions and the extended base node of its cell.
+template <int PM>
+__device__ __forceinline__ int stencil_ext(const RectParams &P, const SliceGeom &G, const float *x, float *w, float *f)
+{
+    int i[3];
+    cell_ext<PM>(P, G, x, i, f);
+    const float2 gxy = __ffma2_rn(make_float2(f[0], f[1]), make_float2(-1.0f, -1.0f), make_float2(1.0f, 1.0f));
+    const float gx = gxy.x, gy = gxy.y, gz = 1.0f - f[2];
+    const float a = gy * gz, b = f[1] * gz, c = gy * f[2], d = f[1] * f[2];
     w[0] = gx * a;
-    w[1] = fx * a;
+    w[1] = f[0] * a;
     w[2] = gx * b;
-    w[3] = fx * b;
+    w[3] = f[0] * b;
     w[4] = gx * c;
-    w[5] = fx * c;
+    w[5] = f[0] * c;
     w[6] = gx * d;
-    w[7] = fx * d;
-    return ix + iy * G.R + iz * (int)G.nxy;
+    w[7] = f[0] * d;
+    return i[0] + i[1] * G.R + i[2] * (int)G.nxy;
 }
 
 // Corner cache: the two z-row quads of the 3 components of the cell a tracer's last stage
@@ -489,88 +541,55 @@ __device__ __forceinline__ void rk4_step3q(const RectParams &P, const SliceGeom 
                                            const float4 *__restrict__ slices, int m0, int m1, int m2, size_t ps,
                                            QuadCache &cc)
 {
-    float k1[3], k2[3], k3[3], k4[3], y[3], w[8];
+    float k1[3], k2[3], k3[3], k4[3], y[3], w[8], f[3];
     const float hh = 0.5f * h;
     const size_t ss = 3 * ps;
     const int nxy = (int)G.nxy;
-    int v = stencil_ext<PM>(P, G, x, w);
+    const auto stage = [&](float c, const float *k) {
+        const float2 q = __ffma2_rn(make_float2(c, c), make_float2(k[0], k[1]), make_float2(x[0], x[1]));
+        y[0] = q.x;
+        y[1] = q.y;
+        y[2] = fmaf(c, k[2], x[2]);
+    };
+    int v = stencil_ext<PM>(P, G, x, w, f);
     interp3q(v, w, slices + (size_t)m0 * ss, m0, ps, nxy, cc, k1);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) y[c] = fmaf(hh, k1[c], x[c]);
-    v = stencil_ext<PM>(P, G, y, w);
+    stage(hh, k1);
+    v = stencil_ext<PM>(P, G, y, w, f);
     interp3q(v, w, slices + (size_t)m1 * ss, m1, ps, nxy, cc, k2);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) y[c] = fmaf(hh, k2[c], x[c]);
-    v = stencil_ext<PM>(P, G, y, w);
+    stage(hh, k2);
+    v = stencil_ext<PM>(P, G, y, w, f);
     interp3q(v, w, slices + (size_t)m1 * ss, m1, ps, nxy, cc, k3);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) y[c] = fmaf(h, k3[c], x[c]);
-    v = stencil_ext<PM>(P, G, y, w);
+    stage(h, k3);
+    v = stencil_ext<PM>(P, G, y, w, f);
     interp3q(v, w, slices + (size_t)m2 * ss, m2, ps, nxy, cc, k4);
     const float h6 = h * (1.0f / 6.0f);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) rk4_advance(x[c], cx[c], h6, k1[c], k2[c], k3[c], k4[c]);
+    float2 xy = make_float2(x[0], x[1]), cxy = make_float2(cx[0], cx[1]);
+    rk4_advance2(xy, cxy, h6, make_float2(k1[0], k1[1]), make_float2(k2[0], k2[1]), make_float2(k3[0], k3[1]),
+                 make_float2(k4[0], k4[1]));
+    x[0] = xy.x;
+    x[1] = xy.y;
+    cx[0] = cxy.x;
+    cx[1] = cxy.y;
+    rk4_advance(x[2], cx[2], h6, k1[2], k2[2], k3[2], k4[2]);
 }
 
 // ------------------------------------------------- variational equations
 
-// stencil_ext plus, for the Jacobian, the fractions and the per-axis factor d s / d x: 1 / h
-// where the query moves with x, 0 on a non-periodic axis where x lies outside the box (the
-// clamped query does not move)
+// u(x) as interp3q and its Jacobian J[c][d] from the same corners (trilinear_grad, as the one-pass variational
+// kernel forms it); on: 1 / h, or 0 on a non-periodic axis where x lies outside the box (the clamped query
+// does not move)
 template <int PM>
-__device__ __forceinline__ int stencil_ext_grad(const RectParams &P, const SliceGeom &G, const float *x, float *w,
-                                                float *f, float *on)
-{
-    int r[3];
-    bool out = false;
-    int ix = axis_cell_ext<PM>(P, G, 0, x[0], f[0], r[0], out);
-    int iy = axis_cell_ext<PM>(P, G, 1, x[1], f[1], r[1], out);
-    int iz = axis_cell_ext<PM>(P, G, 2, x[2], f[2], r[2], out);
-    if (out) {
-        if (per_axis<PM>(P, 0)) ix = wrap_index_slow(r[0], P.n[0]) + G.H[0];
-        if (per_axis<PM>(P, 1)) iy = wrap_index_slow(r[1], P.n[1]) + G.H[1];
-        if (per_axis<PM>(P, 2)) iz = wrap_index_slow(r[2], P.n[2]) + G.H[2];
-    }
-    const float gx = 1.0f - f[0], gy = 1.0f - f[1], gz = 1.0f - f[2];
-    const float a = gy * gz, b = f[1] * gz, c = gy * f[2], d = f[1] * f[2];
-    w[0] = gx * a;
-    w[1] = f[0] * a;
-    w[2] = gx * b;
-    w[3] = f[0] * b;
-    w[4] = gx * c;
-    w[5] = f[0] * c;
-    w[6] = gx * d;
-    w[7] = f[0] * d;
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-        on[k] = (per_axis<PM>(P, k) || (x[k] >= P.origin[k] && x[k] <= P.hi_node[k])) ? P.inv_h[k] : 0.0f;
-    return ix + iy * G.R + iz * (int)G.nxy;
-}
-
-// u(x) as interp3q and its Jacobian J[c][d] = sum_q (d w_q / d x_d) u_q[c], corner q with offsets
-// (q & 1, (q >> 1) & 1, q >> 2), the one-pass variational kernel's products in its order
-__device__ __forceinline__ void interp3q_grad(int v0, const float *w, const float *f, const float *on,
+__device__ __forceinline__ void interp3q_grad(const RectParams &P, const float *x, int v0, const float *w, const float *f,
                                               const float4 *__restrict__ pl, int slice, size_t plane_stride, int nxy,
                                               QuadCache &cc, float *u, float (*J)[3])
 {
+    float on[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        on[k] = (per_axis<PM>(P, k) || (x[k] >= P.origin[k] && x[k] <= P.hi_node[k])) ? P.inv_h[k] : 0.0f;
     interp3q(v0, w, pl, slice, plane_stride, nxy, cc, u);
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            float acc = 0.0f;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                float wq = ((q >> d) & 1) ? 1.0f : -1.0f;
-#pragma unroll
-                for (int e = 0; e < 3; ++e)
-                    if (e != d) wq *= ((q >> e) & 1) ? f[e] : 1.0f - f[e];
-                const float4 qv = cc.q[q >> 2][c];
-                const float uq = (q & 3) == 0 ? qv.x : (q & 3) == 1 ? qv.y : (q & 3) == 2 ? qv.z : qv.w;
-                acc = fmaf(wq, uq, acc);
-            }
-            J[c][d] = acc * on[d];
-        }
+    for (int c = 0; c < 3; ++c) trilinear_grad(cc.q[0][c], cc.q[1][c], f, on, J[c]);
 }
 
 // Steps [s0, min(s1, nsteps)) of every tracer record with the variational equations dM/dt = J M
@@ -609,15 +628,15 @@ __global__ void __launch_bounds__(256, 2) ep_var3_kernel(RectParams P, SliceGeom
             for (int q = 0; q < 4; ++q) {
                 const int sl = ms[q == 0 ? 0 : (q == 3 ? 2 : 1)];
                 const float c = q == 0 ? 0.0f : (q == 3 ? h : hh);
-                float y[3], Y[3][3], w[8], f[3], on[3], J[3][3];
+                float y[3], Y[3][3], w[8], f[3], J[3][3];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     y[a] = q == 0 ? x[a] : fmaf(c, k[q - 1][a], x[a]);
 #pragma unroll
                     for (int b = 0; b < 3; ++b) Y[a][b] = q == 0 ? M[a][b] : fmaf(c, Kp[a][b], M[a][b]);
                 }
-                const int v = stencil_ext_grad<PM>(P, G, y, w, f, on);
-                interp3q_grad(v, w, f, on, slices + (size_t)sl * ss, sl, plane_stride, nxy, cc, k[q], J);
+                const int v = stencil_ext<PM>(P, G, y, w, f);
+                interp3q_grad<PM>(P, y, v, w, f, slices + (size_t)sl * ss, sl, plane_stride, nxy, cc, k[q], J);
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -638,7 +657,7 @@ __global__ void __launch_bounds__(256, 2) ep_var3_kernel(RectParams P, SliceGeom
 #pragma unroll
                 for (int b = 0; b < 3; ++b) M[a][b] = fmaf(h6, S03[a][b] + 2.0f * S12[a][b], M[a][b]);
             }
-            wrap_periodic<3, PM>(P, x, cx, img);
+            wrap_periodic_step<3, PM>(P, x, cx, img);
             if (rect_left<3, PM>(P, x)) {
                 t.st = LCS_TRACER_LEFT;
                 t.te = fmaf((float)(n + 1), h, A.job_t0[job]);
@@ -707,7 +726,7 @@ __global__ void __launch_bounds__(256, LCS_EP_MINB) ep_advect3_kernel(RectParams
         for (int n = s0; n < e; ++n) {
             const int *m = smap + 3 * (n - s0);
             rk4_step3q<PM>(P, G, x, cx, h, slices, __ldg(m), __ldg(m + 1), __ldg(m + 2), plane_stride, cc);
-            wrap_periodic<3, PM>(P, x, cx, img);
+            wrap_periodic_step<3, PM>(P, x, cx, img);
             if (rect_left<3, PM>(P, x)) {
                 t.st = LCS_TRACER_LEFT;
                 t.te = fmaf((float)(n + 1), h, A.job_t0[job]);
@@ -873,7 +892,9 @@ static cudaError_t episodes(const RectParams &P, const lcs_field *f, const Rk4Ar
             lcs_tm_end(L.ctx, 2, s);
             lcs_tm_begin(L.ctx, 0, s);
             // compile-time periodicity for the common all-periodic and non-periodic boxes
-            const int pm = P.periodic[0] | (P.periodic[1] << 1) | (P.periodic[2] << 2);
+            // (of axes within the reach of the kernels' floor)
+            const bool reach = P.n[0] <= FLOOR_MAX_NODES && P.n[1] <= FLOOR_MAX_NODES && P.n[2] <= FLOOR_MAX_NODES;
+            const int pm = reach ? P.periodic[0] | (P.periodic[1] << 1) | (P.periodic[2] << 2) : -1;
             unsigned *kk = last ? nullptr : keys;
             if (var) {
                 if (pm == 7)

@@ -199,6 +199,13 @@ __device__ __forceinline__ void interp_grad(const RectParams &P, const float *x,
         for (int q = 0; q < (1 << DIM); ++q) acc = fmaf(S.w[q], uq[q][c], acc);
         u[c] = acc;
     }
+    if constexpr (DIM == 3) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            trilinear_grad(make_float4(uq[0][c], uq[1][c], uq[2][c], uq[3][c]),
+                           make_float4(uq[4][c], uq[5][c], uq[6][c], uq[7][c]), f, on, J[c]);
+        return;
+    }
     // corner q has offsets (q & 1, (q >> 1) & 1, (q >> 2) & 1); d w_q / d x_d = +-(product of the
     // other axes' weights) / h_d
 #pragma unroll

@@ -399,6 +399,23 @@ __device__ __forceinline__ void interp3p(const Stencil<3> &S, const char *fp, fl
     for (int c = 0; c < 3; ++c) u[c] = acc[c];
 }
 
+// Row of the Jacobian of a trilinear interpolant for one component: a, b its corner values on the two
+// z-faces as (u(0,0), u(1,0), u(0,1), u(1,1)), f the fractions, on the per-axis factor (1 / h, or 0 where the
+// query is clamped).  Differences along an axis interpolated along the other two, both x-corners in one
+// two-lane instruction: 13 of them against 24 multiplications by weight derivatives.
+__device__ __forceinline__ void trilinear_grad(const float4 &a, const float4 &b, const float *f, const float *on, float *J)
+{
+    const float2 m1 = make_float2(-1.0f, -1.0f), fy = make_float2(f[1], f[1]), fz = make_float2(f[2], f[2]);
+    const float2 a0 = make_float2(a.x, a.y), b0 = make_float2(b.x, b.y);
+    const float2 da = __ffma2_rn(a0, m1, make_float2(a.z, a.w)), db = __ffma2_rn(b0, m1, make_float2(b.z, b.w));
+    const float2 ea = __ffma2_rn(fy, da, a0), eb = __ffma2_rn(fy, db, b0);
+    const float2 g = __ffma2_rn(ea, m1, eb);
+    const float2 v = __ffma2_rn(fz, g, ea), dz = __ffma2_rn(fz, __ffma2_rn(da, m1, db), da);
+    J[0] = (v.y - v.x) * on[0];
+    J[1] = fmaf(f[0], dz.y - dz.x, dz.x) * on[1];
+    J[2] = fmaf(f[0], g.y - g.x, g.x) * on[2];
+}
+
 struct Rk4Args {
     const float *seeds;
     long long N;
@@ -490,6 +507,17 @@ __device__ __forceinline__ void wrap_periodic(const RectParams &P, float *x, flo
             }
         }
     }
+}
+
+// wrap_periodic behind one test that the coordinates lie in the box, as they mostly do after a step
+template <int DIM, int PM = -1>
+__device__ __forceinline__ void wrap_periodic_step(const RectParams &P, float *x, float *c, int *img)
+{
+    bool in = true;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d)
+        if (per_axis<PM>(P, d)) in = in && x[d] >= P.origin[d] && x[d] < P.origin[d] + P.L[d];
+    if (!in) wrap_periodic<DIM, PM>(P, x, c, img);
 }
 
 template <int DIM, int PM = -1>
