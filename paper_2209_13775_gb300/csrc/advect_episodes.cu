@@ -16,10 +16,10 @@
 // one-pass kernel.
 //
 // Per episode the field is blended once, in FP32, to every distinct stage time of the
-// episode (a "time slice", stored as xy-quads of the three components interleaved per node, on a
-// lattice with a halo on periodic axes); the advection then reads two 16-byte quads per component and
-// stencil, and keeps the last stencil's corners in registers for the next stage that
-// reads the same slice from the same cell.  FP16/BF16 storage is widened in the fill.
+// episode (a "time slice", on a lattice with a halo on periodic axes; stored as xy-quads of the three
+// components interleaved per node, or as plain nodes where tracers are few); the advection then reads
+// six or eight 16-byte words per stencil, and keeps the last stencil's corners in registers for the next
+// stage that reads the same slice from the same cell.  FP16/BF16 storage is widened in the fill.
 #include "rect_device.cuh"
 
 // Resident 256-thread blocks per SM the advection kernel is compiled for: 4 caps it at
@@ -388,6 +388,44 @@ __global__ void ep_slice_fill_kernel(RectParams P, SliceGeom G, const char *__re
     }
 }
 
+// The second layout: plain nodes (u, v, w, 0), the field blended to the slice's time and nothing repeated.  A
+// stencil is eight 16-byte loads for the quads' six, a slice a third of the bytes to write: for lattices
+// with few tracers per node, where writing the slices costs as much as reading them (slices_plain).  Two
+// x-neighbours in one 32-byte record (four loads, 32 bytes to write) was slower than nodes on sparse
+// lattices and than quads on dense ones (132.4 ms): at eight tracers per node every layout keeps the L1
+// data stage 90% busy, and this one returns a third more bytes than quads.
+template <int ST>
+__global__ void __launch_bounds__(256) ep_node_fill_kernel(RectParams P, SliceGeom G, const char *__restrict__ pairs,
+                                                           size_t fstride, const SchedEntry *__restrict__ stab,
+                                                           const int *__restrict__ nsl, float4 *__restrict__ slices,
+                                                           size_t stride)
+{
+    const long long v = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (v >= G.nodes) return;
+    const int K = (int)(v / G.nxy);
+    const long long rem = v - (long long)K * G.nxy;
+    const int J = (int)(rem / G.R), I = (int)(rem - (long long)J * G.R);
+    if (J >= G.N[1] || I >= G.N[0]) return;
+    const int i = slice_src(I, G.H[0], P.n[0], P.periodic[0]), j = slice_src(J, G.H[1], P.n[1], P.periodic[1]),
+              k = slice_src(K, G.H[2], P.n[2], P.periodic[2]);
+    const int node = (int)(i + j * P.sy + k * P.sz);
+    const int m = __ldg(nsl);
+    float ua[3], ub[3];
+    int kc = -1;
+    for (int q = 0; q < m; ++q) {
+        const SchedEntry e = load_sched(stab + q);
+        if (e.k != kc) {
+            Pair3<ST>::ld(pairs + (size_t)e.k * fstride, node, ua, ub);
+            kc = e.k;
+        }
+        const float g = 1.0f - e.a;
+        float u[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) u[c] = e.a == 0.0f ? ua[c] : tblend(ua[c], ub[c], e.a, g);
+        slices[(size_t)q * stride + v] = make_float4(u[0], u[1], u[2], 0.0f);
+    }
+}
+
 // Cell of x along axis d on the extended lattice, with the fraction f: the same s, floor and
 // f as axis_cell, so the weights are the same.  A periodic index beyond the halo (a stencil
 // point more than SLICE_HALO - 1 cells outside the box) is flagged in `out` and wrapped by
@@ -494,57 +532,72 @@ __device__ __forceinline__ int stencil_ext(const RectParams &P, const SliceGeom 
     return i[0] + i[1] * G.R + i[2] * (int)G.nxy;
 }
 
-// Corner cache: the two z-row quads of the 3 components of the cell a tracer's last stage
-// evaluation read, with the cell's extended base node and the slice they came from.
+// Corner cache: the corner values of the cell a tracer's last stage evaluation read (QUAD: the two z-row quads
+// of the 3 components; NODE: the 8 nodes), with the cell's extended base node and the slice they came from.
 // Stage 3 of an RK4 step reads the same slice as stage 2 (t_n + h/2), and stage 1 of step
 // n + 1 the same slice as stage 4 of step n (t_n + h) whenever the schedule gives both the
 // same (k, alpha); in a smooth flow the second point of each pair is almost always in the
 // same cell as the first, so its corners are already in registers.  The base node fixes
 // all eight corners, so a reuse reads exactly what a reload would: bit-identical results.
-struct QuadCache {
-    float4 q[2][3];
+enum { QUAD = 0, NODE = 1 };
+
+template <int LAY>
+struct CornerCache {
+    float4 q[LAY == QUAD ? 6 : 8];
     int v0;
     int slice;
+    // value of component c at corner k (offsets k & 1, (k >> 1) & 1, k >> 2 along x, y, z)
+    __device__ __forceinline__ float at(int k, int c) const
+    {
+        if constexpr (LAY == QUAD) {
+            const float4 v = q[3 * (k >> 2) + c];
+            return (k & 3) == 0 ? v.x : (k & 3) == 1 ? v.y : (k & 3) == 2 ? v.z : v.w;
+        } else {
+            return c == 0 ? q[k].x : c == 1 ? q[k].y : q[k].z;
+        }
+    }
 };
 
-// u(x) from slice `slice` (3 planes of plane_stride quads at pl); the products and their
-// order are interp3p's: corners (i0,j0,k0), (i1,j0,k0), (i0,j1,k0), (i1,j1,k0), then k1.
+// u(x) from slice `slice` at pl; the products and their order are interp3p's: corners (i0,j0,k0),
+// (i1,j0,k0), (i0,j1,k0), (i1,j1,k0), then k1.
+template <int LAY>
 __device__ __forceinline__ void interp3q(int v0, const float *w, const float4 *__restrict__ pl, int slice,
-                                         size_t plane_stride, int nxy, QuadCache &cc, float *u)
+                                         const SliceGeom &G, CornerCache<LAY> &cc, float *u)
 {
     if (v0 != cc.v0 || slice != cc.slice) {
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
+        for (int r = 0; r < 2; ++r) {
+            const int v = v0 + r * (int)G.nxy;
+            if constexpr (LAY == QUAD) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) cc.q[r][c] = __ldg(pl + 3 * (v0 + r * nxy) + c);
+                for (int c = 0; c < 3; ++c) cc.q[3 * r + c] = __ldg(pl + 3 * v + c);
+            } else {
+                cc.q[4 * r] = __ldg(pl + v);
+                cc.q[4 * r + 1] = __ldg(pl + v + 1);
+                cc.q[4 * r + 2] = __ldg(pl + v + G.R);
+                cc.q[4 * r + 3] = __ldg(pl + v + G.R + 1);
+            }
+        }
         cc.v0 = v0;
         cc.slice = slice;
     }
-    float acc[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
+    for (int c = 0; c < 3; ++c) {
+        float acc = 0.0f;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            acc[c] = fmaf(w[4 * r], cc.q[r][c].x, acc[c]);
-            acc[c] = fmaf(w[4 * r + 1], cc.q[r][c].y, acc[c]);
-            acc[c] = fmaf(w[4 * r + 2], cc.q[r][c].z, acc[c]);
-            acc[c] = fmaf(w[4 * r + 3], cc.q[r][c].w, acc[c]);
-        }
+        for (int k = 0; k < 8; ++k) acc = fmaf(w[k], cc.at(k, c), acc);
+        u[c] = acc;
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) u[c] = acc[c];
 }
 
-// One RK4 step in 3D from slices m0, m1, m2 (stage times t_n, t_n + h/2, t_n + h).
-template <int PM>
+// One RK4 step in 3D from slices m0, m1, m2 (stage times t_n, t_n + h/2, t_n + h), ss quads apart.
+template <int PM, int LAY>
 __device__ __forceinline__ void rk4_step3q(const RectParams &P, const SliceGeom &G, float *x, float *cx, float h,
-                                           const float4 *__restrict__ slices, int m0, int m1, int m2, size_t ps,
-                                           QuadCache &cc)
+                                           const float4 *__restrict__ slices, int m0, int m1, int m2, size_t ss,
+                                           CornerCache<LAY> &cc)
 {
     float k1[3], k2[3], k3[3], k4[3], y[3], w[8], f[3];
     const float hh = 0.5f * h;
-    const size_t ss = 3 * ps;
-    const int nxy = (int)G.nxy;
     const auto stage = [&](float c, const float *k) {
         const float2 q = __ffma2_rn(make_float2(c, c), make_float2(k[0], k[1]), make_float2(x[0], x[1]));
         y[0] = q.x;
@@ -552,16 +605,16 @@ __device__ __forceinline__ void rk4_step3q(const RectParams &P, const SliceGeom 
         y[2] = fmaf(c, k[2], x[2]);
     };
     int v = stencil_ext<PM>(P, G, x, w, f);
-    interp3q(v, w, slices + (size_t)m0 * ss, m0, ps, nxy, cc, k1);
+    interp3q(v, w, slices + (size_t)m0 * ss, m0, G, cc, k1);
     stage(hh, k1);
     v = stencil_ext<PM>(P, G, y, w, f);
-    interp3q(v, w, slices + (size_t)m1 * ss, m1, ps, nxy, cc, k2);
+    interp3q(v, w, slices + (size_t)m1 * ss, m1, G, cc, k2);
     stage(hh, k2);
     v = stencil_ext<PM>(P, G, y, w, f);
-    interp3q(v, w, slices + (size_t)m1 * ss, m1, ps, nxy, cc, k3);
+    interp3q(v, w, slices + (size_t)m1 * ss, m1, G, cc, k3);
     stage(h, k3);
     v = stencil_ext<PM>(P, G, y, w, f);
-    interp3q(v, w, slices + (size_t)m2 * ss, m2, ps, nxy, cc, k4);
+    interp3q(v, w, slices + (size_t)m2 * ss, m2, G, cc, k4);
     const float h6 = h * (1.0f / 6.0f);
     float2 xy = make_float2(x[0], x[1]), cxy = make_float2(cx[0], cx[1]);
     rk4_advance2(xy, cxy, h6, make_float2(k1[0], k1[1]), make_float2(k2[0], k2[1]), make_float2(k3[0], k3[1]),
@@ -578,26 +631,45 @@ __device__ __forceinline__ void rk4_step3q(const RectParams &P, const SliceGeom 
 // u(x) as interp3q and its Jacobian J[c][d] from the same corners (trilinear_grad, as the one-pass variational
 // kernel forms it); on: 1 / h, or 0 on a non-periodic axis where x lies outside the box (the clamped query
 // does not move)
-template <int PM>
-__device__ __forceinline__ void interp3q_grad(const RectParams &P, const float *x, int v0, const float *w, const float *f,
-                                              const float4 *__restrict__ pl, int slice, size_t plane_stride, int nxy,
-                                              QuadCache &cc, float *u, float (*J)[3])
+template <int PM, int LAY>
+__device__ __forceinline__ void interp3q_grad(const RectParams &P, const SliceGeom &G, const float *x, int v0,
+                                              const float *w, const float *f, const float4 *__restrict__ pl, int slice,
+                                              CornerCache<LAY> &cc, float *u, float (*J)[3])
 {
     float on[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
         on[k] = (per_axis<PM>(P, k) || (x[k] >= P.origin[k] && x[k] <= P.hi_node[k])) ? P.inv_h[k] : 0.0f;
-    interp3q(v0, w, pl, slice, plane_stride, nxy, cc, u);
+    interp3q(v0, w, pl, slice, G, cc, u);
+    if constexpr (LAY == QUAD) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) trilinear_grad(cc.q[0][c], cc.q[1][c], f, on, J[c]);
+        for (int c = 0; c < 3; ++c) trilinear_grad(cc.q[c], cc.q[3 + c], f, on, J[c]);
+    } else {
+        // trilinear_grad's operations with u and v (not two x-corners) in the two lanes
+        float2 uv[8], Jp[3];
+        float z[8], Jz[3];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            uv[k] = make_float2(cc.q[k].x, cc.q[k].y);
+            z[k] = cc.q[k].z;
+        }
+        trilinear_grad_nodes(uv, f, on, Jp);
+        trilinear_grad_nodes(z, f, on, Jz);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            J[0][k] = Jp[k].x;
+            J[1][k] = Jp[k].y;
+            J[2][k] = Jz[k];
+        }
+    }
 }
 
 // Steps [s0, min(s1, nsteps)) of every tracer record with the variational equations dM/dt = J M
 // next to Eq. 2: x follows rk4_step3q's arithmetic, M ([9][N] planes, slot-ordered like S) the
 // one-pass variational kernel's, so both match the other paths bit for bit.
-template <int PM>
+template <int PM, int LAY>
 __global__ void __launch_bounds__(256, 2) ep_var3_kernel(RectParams P, SliceGeom G, const float4 *__restrict__ slices,
-                                                        size_t plane_stride, const int *__restrict__ smap, Rk4Args A,
+                                                        size_t ss, const int *__restrict__ smap, Rk4Args A,
                                                         Tracer *__restrict__ S, float *__restrict__ M9, int job,
                                                         int s0, int s1, int shift, unsigned *__restrict__ keys,
                                                         unsigned *__restrict__ hist)
@@ -614,10 +686,8 @@ __global__ void __launch_bounds__(256, 2) ep_var3_kernel(RectParams P, SliceGeom
         for (int e = 0; e < 9; ++e) M[e / 3][e % 3] = M9[e * N + i];
         const int ns = A.job_nsteps[job];
         const float h = A.job_h[job], hh = 0.5f * h, h6 = h * (1.0f / 6.0f);
-        const size_t ss = 3 * plane_stride;
-        const int nxy = (int)G.nxy;
         const int e1 = min(s1, ns);
-        QuadCache cc;
+        CornerCache<LAY> cc;
         cc.v0 = -1;
         cc.slice = -1;
         for (int n = s0; n < e1; ++n) {
@@ -636,7 +706,7 @@ __global__ void __launch_bounds__(256, 2) ep_var3_kernel(RectParams P, SliceGeom
                     for (int b = 0; b < 3; ++b) Y[a][b] = q == 0 ? M[a][b] : fmaf(c, Kp[a][b], M[a][b]);
                 }
                 const int v = stencil_ext<PM>(P, G, y, w, f);
-                interp3q_grad<PM>(P, y, v, w, f, slices + (size_t)sl * ss, sl, plane_stride, nxy, cc, k[q], J);
+                interp3q_grad<PM>(P, G, y, v, w, f, slices + (size_t)sl * ss, sl, cc, k[q], J);
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -702,10 +772,10 @@ __device__ __forceinline__ void ep_store(const RectParams &P, const Rk4Args &A, 
 
 // Steps [s0, min(s1, nsteps)) of every tracer record through the episode's time slices,
 // then the cell key of its new position for the next re-bundling.
-template <int PM>
+template <int PM, int LAY>
 __global__ void __launch_bounds__(256, LCS_EP_MINB) ep_advect3_kernel(RectParams P, SliceGeom G,
                                                                       const float4 *__restrict__ slices,
-                                                                      size_t plane_stride, const int *__restrict__ smap,
+                                                                      size_t ss, const int *__restrict__ smap,
                                                                       Rk4Args A, Tracer *__restrict__ S, int job,
                                                                       int s0, int s1, int shift,
                                                                       unsigned *__restrict__ keys,
@@ -720,12 +790,12 @@ __global__ void __launch_bounds__(256, LCS_EP_MINB) ep_advect3_kernel(RectParams
         const int ns = A.job_nsteps[job];
         const float h = A.job_h[job];
         const int e = min(s1, ns);
-        QuadCache cc;
+        CornerCache<LAY> cc;
         cc.v0 = -1;
         cc.slice = -1;
         for (int n = s0; n < e; ++n) {
             const int *m = smap + 3 * (n - s0);
-            rk4_step3q<PM>(P, G, x, cx, h, slices, __ldg(m), __ldg(m + 1), __ldg(m + 2), plane_stride, cc);
+            rk4_step3q<PM>(P, G, x, cx, h, slices, __ldg(m), __ldg(m + 1), __ldg(m + 2), ss, cc);
             wrap_periodic_step<3, PM>(P, x, cx, img);
             if (rect_left<3, PM>(P, x)) {
                 t.st = LCS_TRACER_LEFT;
@@ -791,11 +861,17 @@ static int sort_shift(long long nodes)
     return shift;
 }
 
-// up to 3 distinct stage times per step, 3 component planes per slice
-static size_t slice_bytes(const SliceGeom &G, int E)
+// Plain nodes rather than quads in the slices: wherever the writes saved outweigh the wider gathers.  RK4,
+// 100 steps on 128^3 nodes, quads / nodes: 0.12 tracers per node 5.86 / 2.99 ms, 1: 9.24 / 7.36, 2: 12.8 /
+// 11.6, 4: 19.5 / 18.8, 8 (400 steps): 129.1 / 131.1.  The variational kernel, bound by issue, gains at any
+// density: 1 per node 12.07 / 9.58 ms, 2: 18.95 / 16.4.
+static bool slices_plain(const lcs_field *f, long long N, bool var) { return var || N < 6 * f->nodes; }
+
+// up to 3 distinct stage times per step; quads: 48 bytes per node, plain nodes: 16
+static size_t slice_bytes(const SliceGeom &G, int E, bool plain)
 {
-    return al256(16 * (size_t)G.nodes) * 9 * E + al256(sizeof(int) * 3 * E) + al256(sizeof(SchedEntry) * 3 * E) +
-           256;
+    return al256(16 * (size_t)G.nodes) * (plain ? 3 : 9) * E + al256(sizeof(int) * 3 * E) +
+           al256(sizeof(SchedEntry) * 3 * E) + 256;
 }
 
 size_t rk4_sorted_scratch_bytes(long long N, const lcs_field *f, int E, bool variational)
@@ -804,7 +880,7 @@ size_t rk4_sorted_scratch_bytes(long long N, const lcs_field *f, int E, bool var
     long long nbins = ((keys - 1) >> sort_shift(keys)) + 1;
     long long nb = (nbins + SCAN_TILE - 1) / SCAN_TILE;
     size_t b = 2 * al256(sizeof(Tracer) * N) + 2 * al256(4 * N) + 2 * al256(4 * nbins) + al256(4 * nb);
-    b += slice_bytes(slice_geom(f), E);
+    b += slice_bytes(slice_geom(f), E, slices_plain(f, N, variational));
     if (variational) b += 2 * al256(sizeof(float) * 9 * N);   // grad F planes, ping-pong with the records
     return b;
 }
@@ -838,24 +914,25 @@ static cudaError_t episodes(const RectParams &P, const lcs_field *f, const Rk4Ar
     const SliceGeom G = slice_geom(f);
     if (G.nodes > (1LL << 30)) return cudaErrorInvalidValue;
     const size_t plane_stride = al256(16 * (size_t)G.nodes) / 16;
+    const bool var = A.out_grad != nullptr, plain = slices_plain(f, N, var);
     float4 *slices = nullptr;
     int *smap = nullptr, *nsl = nullptr;
     SchedEntry *stab = nullptr;
     {
         slices = (float4 *)p;
-        p += al256(16 * (size_t)G.nodes) * 9 * E;
+        p += al256(16 * (size_t)G.nodes) * (plain ? 3 : 9) * E;
         smap = (int *)p;
         p += al256(sizeof(int) * 3 * E);
         stab = (SchedEntry *)p;
         p += al256(sizeof(SchedEntry) * 3 * E);
         nsl = (int *)p;
+        p += 256;
     }
     // variational grad F: [9][N] planes after the rest of the working memory, moved with the records
-    const bool var = A.out_grad != nullptr;
     float *MA = nullptr, *MB = nullptr;
     if (var) {
-        MA = (float *)((char *)L.work + rk4_sorted_scratch_bytes(N, f, E, false));
-        MB = (float *)((char *)MA + al256(sizeof(float) * 9 * N));
+        MA = (float *)p;
+        MB = (float *)(p + al256(sizeof(float) * 9 * N));
     }
     const int bt = 256;
     const unsigned grid = (unsigned)((N + bt - 1) / bt);
@@ -887,8 +964,14 @@ static cudaError_t episodes(const RectParams &P, const lcs_field *f, const Rk4Ar
             lcs_tm_end(L.ctx, 1, s);
             lcs_tm_begin(L.ctx, 2, s);
             ep_slice_table_kernel<<<1, 32, 0, s>>>(A.sched, A.nsteps_max, job, s0, s1, smap, stab, nsl);
-            ep_slice_fill_kernel<ST><<<(unsigned)((G.nodes + 255) / 256), 256, 0, s>>>(
-                P, G, (const char *)f->d_frames, f->frame_stride, stab, nsl, slices, plane_stride);
+            const unsigned fgrid = (unsigned)((G.nodes + 255) / 256);
+            const size_t ss = plain ? plane_stride : 3 * plane_stride;   // quads from slice to slice
+            if (plain)
+                ep_node_fill_kernel<ST><<<fgrid, 256, 0, s>>>(P, G, (const char *)f->d_frames, f->frame_stride, stab, nsl,
+                                                              slices, ss);
+            else
+                ep_slice_fill_kernel<ST><<<fgrid, 256, 0, s>>>(P, G, (const char *)f->d_frames, f->frame_stride, stab, nsl,
+                                                               slices, plane_stride);
             lcs_tm_end(L.ctx, 2, s);
             lcs_tm_begin(L.ctx, 0, s);
             // compile-time periodicity for the common all-periodic and non-periodic boxes
@@ -896,25 +979,27 @@ static cudaError_t episodes(const RectParams &P, const lcs_field *f, const Rk4Ar
             const bool reach = P.n[0] <= FLOOR_MAX_NODES && P.n[1] <= FLOOR_MAX_NODES && P.n[2] <= FLOOR_MAX_NODES;
             const int pm = reach ? P.periodic[0] | (P.periodic[1] << 1) | (P.periodic[2] << 2) : -1;
             unsigned *kk = last ? nullptr : keys;
-            if (var) {
-                if (pm == 7)
-                    ep_var3_kernel<7><<<agrid, abt, 0, s>>>(P, G, slices, plane_stride, smap, A, SB, MB, job, s0, s1,
-                                                           shift, kk, hist);
-                else if (pm == 0)
-                    ep_var3_kernel<0><<<agrid, abt, 0, s>>>(P, G, slices, plane_stride, smap, A, SB, MB, job, s0, s1,
-                                                           shift, kk, hist);
-                else
-                    ep_var3_kernel<-1><<<agrid, abt, 0, s>>>(P, G, slices, plane_stride, smap, A, SB, MB, job, s0,
-                                                            s1, shift, kk, hist);
-            } else if (pm == 7)
-                ep_advect3_kernel<7><<<agrid, abt, 0, s>>>(P, G, slices, plane_stride, smap, A, SB, job, s0, s1, shift,
-                                                          kk, hist);
-            else if (pm == 0)
-                ep_advect3_kernel<0><<<agrid, abt, 0, s>>>(P, G, slices, plane_stride, smap, A, SB, job, s0, s1, shift,
-                                                          kk, hist);
+#define EP_VAR(PM, LAY) \
+    ep_var3_kernel<PM, LAY><<<agrid, abt, 0, s>>>(P, G, slices, ss, smap, A, SB, MB, job, s0, s1, shift, kk, hist)
+#define EP_ADV(PM, LAY) \
+    ep_advect3_kernel<PM, LAY><<<agrid, abt, 0, s>>>(P, G, slices, ss, smap, A, SB, job, s0, s1, shift, kk, hist)
+#define EP_LAUNCH(K)                                \
+    do {                                            \
+        if (pm == 7) {                              \
+            if (plain) K(7, NODE); else K(7, QUAD); \
+        } else if (pm == 0) {                       \
+            if (plain) K(0, NODE); else K(0, QUAD); \
+        } else {                                    \
+            if (plain) K(-1, NODE); else K(-1, QUAD); \
+        }                                           \
+    } while (0)
+            if (var)
+                EP_LAUNCH(EP_VAR);
             else
-                ep_advect3_kernel<-1><<<agrid, abt, 0, s>>>(P, G, slices, plane_stride, smap, A, SB, job, s0, s1,
-                                                           shift, kk, hist);
+                EP_LAUNCH(EP_ADV);
+#undef EP_VAR
+#undef EP_ADV
+#undef EP_LAUNCH
             lcs_tm_end(L.ctx, 0, s);
             if (snap_out >= 0)
                 ep_snapshot_kernel<<<grid, bt, 0, s>>>(P, SB, A, snap_out, snap_out - L.njobs);

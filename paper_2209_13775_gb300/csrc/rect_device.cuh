@@ -416,6 +416,30 @@ __device__ __forceinline__ void trilinear_grad(const float4 &a, const float4 &b,
     J[2] = fmaf(f[0], g.y - g.x, g.x) * on[2];
 }
 
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float2 vfma(float a, float2 b, float2 c) { return __ffma2_rn(make_float2(a, a), b, c); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float a, float2 b) { return __fmul2_rn(make_float2(a, a), b); }
+
+// trilinear_grad's operations on the eight corner values u[k] (offsets k & 1, (k >> 1) & 1, k >> 2) of one
+// component (V = float) or of two (float2): the same bits
+template <class V>
+__device__ __forceinline__ void trilinear_grad_nodes(const V *u, const float *f, const float *on, V *J)
+{
+    V v[2], dz[2], g[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {   // the two x-corners
+        const V da = vfma(-1.0f, u[i], u[2 + i]), db = vfma(-1.0f, u[4 + i], u[6 + i]);
+        const V ea = vfma(f[1], da, u[i]), eb = vfma(f[1], db, u[4 + i]);
+        g[i] = vfma(-1.0f, ea, eb);
+        v[i] = vfma(f[2], g[i], ea);
+        dz[i] = vfma(f[2], vfma(-1.0f, da, db), da);
+    }
+    J[0] = vmul(on[0], vfma(-1.0f, v[0], v[1]));
+    J[1] = vmul(on[1], vfma(f[0], vfma(-1.0f, dz[0], dz[1]), dz[0]));
+    J[2] = vmul(on[2], vfma(f[0], vfma(-1.0f, g[0], g[1]), g[0]));
+}
+
 struct Rk4Args {
     const float *seeds;
     long long N;
