@@ -570,65 +570,58 @@ __device__ __forceinline__ bool same_slice(SchedEntry a, SchedEntry b)
            (b.k + 1 == a.k && b.a == 1.0f && a.a == 0.0f);
 }
 
-// shared[job][n] = 1 where step n of the job starts at the time its step n - 1 ended, and so needs no first
-// slice of its own
-__global__ void slice2d_shared_kernel(const SchedEntry *__restrict__ sched, int nsteps_max, int njobs,
-                                      unsigned char *__restrict__ shared)
+// A thread fills its node in FILL_RUN consecutive slices of a job (blocks: nodes x runs x jobs), so the node's
+// corners are found once and the frames they are blended from are loaded once per bracket.  shared[job][n] = 1
+// where step n starts at the time its step n - 1 ended: that step has no first slice of its own.
+#define FILL_RUN 12
+template <int ST>
+__global__ void __launch_bounds__(256) slice2d_fill_kernel(RectParams P, const char *__restrict__ frames, size_t fstride,
+                                                           const SchedEntry *__restrict__ sched, int nsteps_max,
+                                                           const int *__restrict__ job_nsteps,
+                                                           const __grid_constant__ Slice2dOffsets O, int nodes,
+                                                           unsigned char *__restrict__ shared,
+                                                           float4 *__restrict__ slices)
 {
-    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (t >= (long long)njobs * nsteps_max) return;
-    shared[t] = t % nsteps_max > 0 && same_slice(load_sched(sched + 3 * t - 1), load_sched(sched + 3 * t));
-}
-
-__global__ void slice2d_fill_kernel(RectParams P, const char *__restrict__ frames, size_t fstride, int storage,
-                                    const SchedEntry *__restrict__ sched, int nsteps_max,
-                                    const int *__restrict__ job_nsteps, Slice2dOffsets O, long long nodes,
-                                    const unsigned char *__restrict__ shared, float4 *__restrict__ slices)
-{
-    const int job = blockIdx.y;
-    const unsigned char *sh = shared + (size_t)job * nsteps_max;
-    const long long per_job = 3LL * job_nsteps[job] * nodes;
+    const int job = blockIdx.z, v = blockIdx.x * 256 + threadIdx.x;
+    const long long nsl = 3LL * job_nsteps[job];
+    if (v >= nodes) return;
     const SchedEntry *sc = sched + (size_t)job * nsteps_max * 3;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < per_job;
-         t += (long long)gridDim.x * blockDim.x) {
-        const long long l = t / nodes, v = t % nodes;
-        if (l % 3 == 0 && sh[l / 3]) continue;     // the last slice of the step before serves
+    const int j = v / P.n[0], i = v - j * P.n[0];
+    const int i1 = P.periodic[0] ? (i + 1 == P.n[0] ? 0 : i + 1) : min(i + 1, P.n[0] - 1);
+    const int j1 = P.periodic[1] ? (j + 1 == P.n[1] ? 0 : j + 1) : min(j + 1, P.n[1] - 1);
+    const int sy = (int)P.sy, corner[4] = {i + j * sy, i1 + j * sy, i + j1 * sy, i1 + j1 * sy};
+    float ua[4][2], ub[4][2];
+    int ka = -1, kb = -1;
+    // (one run per block unless a job has more runs than a grid has rows)
+    for (long long l = (long long)blockIdx.y * FILL_RUN; l < nsl;
+         l += (l + 1) % FILL_RUN ? 1 : (gridDim.y - 1) * (long long)FILL_RUN + 1) {
         const SchedEntry e = load_sched(sc + l);   // slice l of the job = schedule entry l (= 3 n + stage)
-        const int i = (int)(v % P.n[0]), j = (int)(v / P.n[0]);
-        const int i1 = P.periodic[0] ? (i + 1 == P.n[0] ? 0 : i + 1) : min(i + 1, P.n[0] - 1);
-        const int j1 = P.periodic[1] ? (j + 1 == P.n[1] ? 0 : j + 1) : min(j + 1, P.n[1] - 1);
-        const int corner[4] = {(int)(i + j * P.sy), (int)(i1 + j * P.sy), (int)(i + j1 * P.sy),
-                               (int)(i1 + j1 * P.sy)};
-        const char *fa = frames + (size_t)e.k * fstride;
-        float u[4][2];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            float va[2], vb[2];
-            if (storage == LCS_F32)
-                Node<2, LCS_F32>::ld(fa, corner[q], va);
-            else if (storage == LCS_F16)
-                Node<2, LCS_F16>::ld(fa, corner[q], va);
-            else
-                Node<2, LCS_BF16>::ld(fa, corner[q], va);
-            if (e.a == 0.0f) {   // frame k + 1 is not read (it may not exist)
-                u[q][0] = va[0];
-                u[q][1] = va[1];
-                continue;
-            }
-            const char *fb = fa + fstride;
-            if (storage == LCS_F32)
-                Node<2, LCS_F32>::ld(fb, corner[q], vb);
-            else if (storage == LCS_F16)
-                Node<2, LCS_F16>::ld(fb, corner[q], vb);
-            else
-                Node<2, LCS_BF16>::ld(fb, corner[q], vb);
-            const float g = 1.0f - e.a;
-            u[q][0] = tblend(va[0], vb[0], e.a, g);
-            u[q][1] = tblend(va[1], vb[1], e.a, g);
+        if (l % 3 == 0) {
+            const bool same = l > 0 && same_slice(load_sched(sc + l - 1), e);
+            if (v == 0) shared[(size_t)job * nsteps_max + l / 3] = same;
+            if (same) continue;                    // the last slice of the step before serves
         }
-        float4 *o = slices + (O.off[job] + l) * 2 * nodes + 2 * v;
-        o[0] = make_float4(u[0][0], u[1][0], u[2][0], u[3][0]);
-        o[1] = make_float4(u[0][1], u[1][1], u[2][1], u[3][1]);
+        const char *fa = frames + (size_t)e.k * fstride;
+        if (e.k != ka) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) Node<2, ST>::ld(fa, corner[q], ua[q]);
+            ka = e.k;
+        }
+        if (e.a != 0.0f && e.k != kb) {            // frame k + 1 is not read at weight 0 (it may not exist)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) Node<2, ST>::ld(fa + fstride, corner[q], ub[q]);
+            kb = e.k;
+        }
+        const float g = 1.0f - e.a;
+        float u[2][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) u[c][q] = e.a == 0.0f ? ua[q][c] : tblend(ua[q][c], ub[q][c], e.a, g);
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(slices + ((O.off[job] + l) * nodes + v) * 2),
+                     "f"(u[0][0]), "f"(u[0][1]), "f"(u[0][2]), "f"(u[0][3]), "f"(u[1][0]), "f"(u[1][1]), "f"(u[1][2]),
+                     "f"(u[1][3])
+                     : "memory");
     }
 }
 
@@ -728,6 +721,32 @@ __device__ __forceinline__ float2 interp2s_box(const Box2 &B, float2 x, const ch
                        fmaf(w[3], q[7], fmaf(w[2], q[6], fmaf(w[1], q[5], fmaf(w[0], q[4], 0.0f)))));
 }
 
+// The record of the cell that p lies in, and those of its neighbours that p comes near, into the L1 cache: four
+// bytes of each by an asynchronous copy to shared memory, which allocates the record's sector on its way
+// (prefetch.global.L1 has no effect here) and holds up nobody.  sl as in interp2s_box, last: box2_cell's id of
+// the slice's last node (every id read is clamped to the slice).
+__device__ __forceinline__ void records_ahead(const Box2 &B, float2 p, const char *sl, float last, uint32_t sink)
+{
+    const float2 s = __fmul2_rn(__fadd2_rn(p, B.no), B.inv);
+    float2 t = __fadd2_rd(s, make_float2(FLOOR_MAGIC, FLOOR_MAGIC));
+    t = make_float2(fminf(fmaxf(t.x, FLOOR_MAGIC), B.tmax.x), fminf(fmaxf(t.y, FLOOR_MAGIC), B.tmax.y));
+    const float fx = s.x - (t.x - FLOOR_MAGIC), fy = s.y - (t.y - FLOOR_MAGIC);
+    const float id = fmaf(FLOOR_MAGIC - t.y, B.nnx, t.x);
+    const float dx = fx < 0.5f ? -1.0f : 1.0f, dy = fy < 0.5f ? B.nnx : -B.nnx;
+    const bool nx = fabsf(fx - 0.5f) > 0.3f, ny = fabsf(fy - 0.5f) > 0.3f;
+    const auto take = [&](float i, bool on) {
+        const char *q = sl + 32LL * __float_as_int(fminf(fmaxf(i, FLOOR_MAGIC), last));
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p cp.async.ca.shared.global [%0], [%1], 4;\n\t}" ::"r"(sink),
+            "l"(q), "r"((unsigned)on)
+            : "memory");
+    };
+    take(id, true);
+    take(id + dx, nx);
+    take(id + dy, ny);
+    take(id + dx + dy, nx && ny);
+}
+
 // rk4_slice2d_kernel on a closed box (box2_ok).  Issue bounds it on large lattices (176 warp-instructions per
 // step of 213 before), so the cell, the stage points and the update run in two-lane FP32 instructions, the
 // cell without the conversion pipe, and a stencil is one load; load latency bounds it on small ones, so the
@@ -735,7 +754,7 @@ __device__ __forceinline__ float2 interp2s_box(const Box2 &B, float2 x, const ch
 // their point is in its cell (L1 sectors 655 M -> 201 M on four windows).  The same operations in the same
 // order: the same bits.  64 windows of 2048 x 1024 seeds: 78.8 -> 73.1 ms; 64 x 32 seeds, 100 steps: 191 ->
 // 151 us.  All-scalar arithmetic: 76.3 ms; 40 registers (six blocks): 76.1 ms.
-template <bool UNIT>
+template <bool UNIT, bool AHEAD>
 __global__ void __launch_bounds__(256) rk4_slice2d_box_kernel(const __grid_constant__ RectParams P,
                                                               const __grid_constant__ Box2 B,
                                                               const float4 *__restrict__ slices, long long nodes,
@@ -761,6 +780,11 @@ __global__ void __launch_bounds__(256) rk4_slice2d_box_kernel(const __grid_const
         store_tracer<2>(P, A, slot, i, xs, cs, img, st, t_exit);
     };
     const unsigned char *sh = shared + (size_t)job * A.nsteps_max;
+    __shared__ unsigned int sink_words[AHEAD ? 256 : 1];   // where copies for the cache's sake go; never read
+    const uint32_t sink = smem_u32(sink_words + (AHEAD ? threadIdx.x : 0));
+    const float last = FLOOR_MAGIC + (float)(nodes - 1);
+    float2 kp = make_float2(0.0f, 0.0f);                   // first slope of the step before
+    bool first = true;
     RecordCache cc;
     cc.v = -1;
 #pragma unroll
@@ -771,6 +795,16 @@ __global__ void __launch_bounds__(256) rk4_slice2d_box_kernel(const __grid_const
         const bool kept = __ldg(sh + n) != 0;
         if (!kept) cc.v = -1;
         const float2 k1 = interp2s_box<UNIT, true>(B, x, kept ? s0 - ss : s0, cc);
+        if (AHEAD && first) kp = k1;
+        first = false;
+        if (AHEAD && n + 1 < ns) {   // where the next step's second and fourth stage will be, to second order
+            const float2 dk = make_float2(k1.x - kp.x, k1.y - kp.y);
+            records_ahead(B, make_float2(fmaf(1.125f * h, dk.x, fmaf(1.5f * h, k1.x, x.x)),
+                                         fmaf(1.125f * h, dk.y, fmaf(1.5f * h, k1.y, x.y))), s0 + 4 * ss, last, sink);
+            records_ahead(B, make_float2(fmaf(2.0f * h, dk.x, fmaf(2.0f * h, k1.x, x.x)),
+                                         fmaf(2.0f * h, dk.y, fmaf(2.0f * h, k1.y, x.y))), s0 + 5 * ss, last, sink);
+            kp = k1;
+        }
         const float2 k2 = interp2s_box<UNIT, false>(B, __ffma2_rn(h2, k1, x), s0 + ss, cc);
         const float2 k3 = interp2s_box<UNIT, true>(B, __ffma2_rn(h2, k2, x), s0 + ss, cc);
         const float2 k4 = interp2s_box<UNIT, false>(B, __ffma2_rn(make_float2(h, h), k3, x), s0 + 2 * ss, cc);
@@ -785,6 +819,7 @@ __global__ void __launch_bounds__(256) rk4_slice2d_box_kernel(const __grid_const
             next = ++si < A.nsnap ? snap_step(A, si, ns) : -1;
         }
     }
+    if (AHEAD) asm volatile("cp.async.wait_all;" ::: "memory");
     for (; si < A.nsnap; ++si) store(snap_slot(A, job, si), snap_exit(A, job, si, st, te));
     store(job, te);
 }
@@ -812,21 +847,34 @@ static cudaError_t launch_slice2d(const RectParams &P, const lcs_field *f, const
     float4 *slices = (float4 *)L.work;
     const long long nodes = f->nodes;
     unsigned char *shared = (unsigned char *)(slices + acc * 2 * nodes);
-    const long long flags = (long long)L.njobs * A.nsteps_max;
-    lcs_tm_begin(L.ctx, 2, s);
-    if (flags > 0)
-        slice2d_shared_kernel<<<(unsigned)((flags + 255) / 256), 256, 0, s>>>(A.sched, A.nsteps_max, L.njobs, shared);
-    slice2d_fill_kernel<<<dim3(1024, (unsigned)L.njobs), 256, 0, s>>>(P, (const char *)f->d_frames, f->frame_stride,
-                                                                      f->storage, A.sched, A.nsteps_max,
-                                                                      A.job_nsteps, O, nodes, shared, slices);
+    if (A.nsteps_max > 0) {
+        const long long runs = (3LL * A.nsteps_max + FILL_RUN - 1) / FILL_RUN;
+        const dim3 fgrid((unsigned)((nodes + 255) / 256), (unsigned)(runs < 65535 ? runs : 65535), (unsigned)L.njobs);
+        const char *fr = (const char *)f->d_frames;
+#define FILL(ST)                                                                                                      \
+    slice2d_fill_kernel<ST><<<fgrid, 256, 0, s>>>(P, fr, f->frame_stride, A.sched, A.nsteps_max, A.job_nsteps, O,    \
+                                                  (int)nodes, shared, slices)
+        if (f->storage == LCS_F32) FILL(LCS_F32);
+        else if (f->storage == LCS_F16) FILL(LCS_F16);
+        else FILL(LCS_BF16);
+#undef FILL
+    }
     lcs_tm_end(L.ctx, 2, s);
     lcs_tm_begin(L.ctx, 0, s);
     dim3 grid(seed_map_grid(A.map, A.N, bt), (unsigned)L.njobs);
     const int pm = P.periodic[0] | (P.periodic[1] << 1);
-    if (box2_ok(P) && box2_unit(P))
-        rk4_slice2d_box_kernel<true><<<grid, bt, 0, s>>>(P, make_box2(P), slices, nodes, O, shared, A);
+    // up to eight warps per SM the steps of a tracer wait for one L2 round trip after another, and copying the
+    // records of the step after next ahead pays: 100 steps of 64 x 32 seeds 146 -> 106 us, of 256 x 128 127 ->
+    // 100; of 400 x 200 (16 warps per SM) it would cost (126 -> 146)
+    const bool ahead = A.N * L.njobs <= 256LL * L.ctx->num_sms;
+    if (box2_ok(P) && box2_unit(P) && ahead)
+        rk4_slice2d_box_kernel<true, true><<<grid, bt, 0, s>>>(P, make_box2(P), slices, nodes, O, shared, A);
+    else if (box2_ok(P) && ahead)
+        rk4_slice2d_box_kernel<false, true><<<grid, bt, 0, s>>>(P, make_box2(P), slices, nodes, O, shared, A);
+    else if (box2_ok(P) && box2_unit(P))
+        rk4_slice2d_box_kernel<true, false><<<grid, bt, 0, s>>>(P, make_box2(P), slices, nodes, O, shared, A);
     else if (box2_ok(P))
-        rk4_slice2d_box_kernel<false><<<grid, bt, 0, s>>>(P, make_box2(P), slices, nodes, O, shared, A);
+        rk4_slice2d_box_kernel<false, false><<<grid, bt, 0, s>>>(P, make_box2(P), slices, nodes, O, shared, A);
     else if (pm == 3)
         rk4_slice2d_kernel<3><<<grid, bt, 0, s>>>(P, slices, nodes, O, shared, A);
     else
@@ -996,7 +1044,10 @@ int launch_rk4_rect(lcs_ctx *ctx, const Rk4Launch &L, cudaStream_t s)
         return e == cudaSuccess ? variant : -1;
     }
     if (variant == 5) {
-        int bt = L.block_threads > 0 && L.block_threads <= 256 ? L.block_threads : 256;
+        // few tracers: one warp per block spreads them over the SMs (64 x 32 seeds: 106 us, 145 in blocks of 256)
+        int bt = L.block_threads > 0 && L.block_threads <= 256 ? L.block_threads
+                 : A.N * L.njobs <= 64LL * ctx->num_sms         ? 32
+                                                                 : 256;
         A.map = make_seed_map(L.lat_dim, L.lat_n, bt);
         e = launch_slice2d(P, f, A, L, bt, s);
         return e == cudaSuccess ? variant : -1;
