@@ -113,10 +113,11 @@ cudaError_t launch_rk4_schedule(const double *d_times, int nframes, int time_per
 
 // ============================================================ gather kernel
 
-template <int DIM, int ST>
-__global__ void __launch_bounds__(256) rk4_gather_kernel(RectParams P, const char *__restrict__ frames,
-                                                         size_t fstride, Rk4Args A)
+template <int ST>
+__global__ void __launch_bounds__(256) rk4_gather2_kernel(RectParams P, const char *__restrict__ frames,
+                                                          size_t fstride, Rk4Args A)
 {
+    constexpr int DIM = 2;
     const long long i = thread_tracer(A);
     int job = blockIdx.y;
     if (i < 0) return;
@@ -137,14 +138,10 @@ __global__ void __launch_bounds__(256) rk4_gather_kernel(RectParams P, const cha
     int si = 0;   // next snapshot
     for (int n = 0; n < ns; ++n) {
         SchedEntry e0 = load_sched(sc + 3 * n), e1 = load_sched(sc + 3 * n + 1), e2 = load_sched(sc + 3 * n + 2);
-        if constexpr (DIM == 2)
-            rk4_step<2, ST, SRC_GLOBAL>(P, x, cx, h, frames + (size_t)e0.k * fstride,
-                                        frames + (size_t)(e0.k + 1) * fstride, e0.a, frames + (size_t)e1.k * fstride,
-                                        frames + (size_t)(e1.k + 1) * fstride, e1.a, frames + (size_t)e2.k * fstride,
-                                        frames + (size_t)(e2.k + 1) * fstride, e2.a);
-        else
-            rk4_step3p<ST>(P, x, cx, h, frames + (size_t)e0.k * fstride, e0.a, frames + (size_t)e1.k * fstride,
-                           e1.a, frames + (size_t)e2.k * fstride, e2.a);
+        rk4_step<2, ST, SRC_GLOBAL>(P, x, cx, h, frames + (size_t)e0.k * fstride,
+                                    frames + (size_t)(e0.k + 1) * fstride, e0.a, frames + (size_t)e1.k * fstride,
+                                    frames + (size_t)(e1.k + 1) * fstride, e1.a, frames + (size_t)e2.k * fstride,
+                                    frames + (size_t)(e2.k + 1) * fstride, e2.a);
         wrap_periodic<DIM>(P, x, cx, img);
         if (rect_left<DIM>(P, x)) {
             st = LCS_TRACER_LEFT;
@@ -159,78 +156,234 @@ __global__ void __launch_bounds__(256) rk4_gather_kernel(RectParams P, const cha
     store_tracer<DIM>(P, A, job, i, x, cx, img, st, te);
 }
 
+// ------------------------------------------------------------ 3D gather
+
+// Cell i0 (each axis' lower node) and fraction f of x, as axis_cell gives them.  PM >= 0 (boxes whose axes all
+// wrap, or all end, of at most FLOOR_MAX_NODES nodes): the floor without the conversion pipe, x and y in
+// two-lane FP32 instructions; indices more than a period away, which include every coordinate beyond the
+// reach of that floor, go back to floorf.
+template <int PM>
+__device__ __forceinline__ void cell3(const RectParams &P, const float *x, int *i0, float *f)
+{
+    if constexpr (PM >= 0) {
+        const float2 M2 = make_float2(FLOOR_MAGIC, FLOOR_MAGIC), m1 = make_float2(-1.0f, -1.0f);
+        float2 q = make_float2(x[0], x[1]);
+        float z = x[2];
+        if constexpr (PM == 0) {
+            q.x = fminf(fmaxf(q.x, P.origin[0]), P.hi_node[0]);
+            q.y = fminf(fmaxf(q.y, P.origin[1]), P.hi_node[1]);
+            z = fminf(fmaxf(z, P.origin[2]), P.hi_node[2]);
+        }
+        const float2 s = __fmul2_rn(__fadd2_rn(q, make_float2(-P.origin[0], -P.origin[1])),
+                                    make_float2(P.inv_h[0], P.inv_h[1]));
+        const float sz = __fmul_rn(z - P.origin[2], P.inv_h[2]);
+        float2 t = __fadd2_rd(s, M2);
+        float tz = __fadd_rd(sz, FLOOR_MAGIC);
+        if constexpr (PM == 0) {
+            t.x = fminf(t.x, FLOOR_MAGIC + (float)(P.n[0] - 2));
+            t.y = fminf(t.y, FLOOR_MAGIC + (float)(P.n[1] - 2));
+            tz = fminf(tz, FLOOR_MAGIC + (float)(P.n[2] - 2));
+        }
+        const float2 fr = __fadd2_rn(s, __ffma2_rn(t, m1, M2));
+        f[0] = fr.x;
+        f[1] = fr.y;
+        f[2] = __fsub_rn(sz, tz - FLOOR_MAGIC);
+        i0[0] = floor_index(t.x);
+        i0[1] = floor_index(t.y);
+        i0[2] = floor_index(tz);
+        if constexpr (PM == 7) {
+            const float sd[3] = {s.x, s.y, sz};
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int n = P.n[d], i = i0[d];
+                int w = i < 0 ? i + n : (i >= n ? i - n : i);
+                if ((unsigned)w >= (unsigned)n) {
+                    const float fl = floorf(sd[d]);
+                    f[d] = sd[d] - fl;
+                    w = wrap_index_slow((int)fl, n);
+                }
+                i0[d] = w;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            int i1;
+            axis_cell<PM>(P, d, x[d], i0[d], i1, f[d]);
+        }
+    }
+}
+
+// periodicity mask of a 3D box whose axes lie within the reach of cell3's floor, or -1
+static int box3_mask(const RectParams &P)
+{
+    for (int d = 0; d < 3; ++d)
+        if (P.n[d] > FLOOR_MAX_NODES) return -1;
+    return (P.periodic[0] ? 1 : 0) | (P.periodic[1] ? 2 : 0) | (P.periodic[2] ? 4 : 0);
+}
+
+// The corners of a tracer's last cell, blended to the time of its last stage (k, a)
+struct BlendCache {
+    float u[8][3];
+    int v0, k;
+    float a;
+};
+
+// u(x) at schedule entry e: interp3p's values.  Stage 3 of a step shares the time of stage 2 and stage 1 mostly
+// that of the stage 4 before, and their points are mostly in the same cells, so half of the stencils need no
+// loads, conversions or blends.
+template <int ST, int PM>
+__device__ __forceinline__ void interp3_cached(const RectParams &P, const float *x, const char *__restrict__ frames,
+                                               size_t fstride, SchedEntry e, BlendCache &cc, float *f, float *u)
+{
+    int i[3];
+    cell3<PM>(P, x, i, f);
+    const int sy = (int)P.sy, sz = (int)P.sz, v0 = i[0] + i[1] * sy + i[2] * sz;
+    if (v0 != cc.v0 || e.k != cc.k || e.a != cc.a) {
+        int dx[3] = {1, sy, sz};   // to the upper node of each axis
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            if (per_axis<PM>(P, d) && i[d] + 1 == P.n[d]) dx[d] -= P.n[d] * dx[d];
+        const char *fp = frames + (size_t)e.k * fstride;
+        const float g = 1.0f - e.a;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            float va[3], vb[3];
+            Pair3<ST>::ld(fp, v0 + (q & 1 ? dx[0] : 0) + (q & 2 ? dx[1] : 0) + (q & 4 ? dx[2] : 0), va, vb);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) cc.u[q][c] = e.a == 0.0f ? va[c] : tblend(va[c], vb[c], e.a, g);
+        }
+        cc.v0 = v0;
+        cc.k = e.k;
+        cc.a = e.a;
+    }
+    const float gx = 1.0f - f[0], gy = 1.0f - f[1], gz = 1.0f - f[2];
+    const float a = gy * gz, b = f[1] * gz, c = gy * f[2], d = f[1] * f[2];
+    const float w[8] = {gx * a, f[0] * a, gx * b, f[0] * b, gx * c, f[0] * c, gx * d, f[0] * d};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        float acc = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc = fmaf(w[q], cc.u[q][k], acc);
+        u[k] = acc;
+    }
+}
+
+// One pass over a job's steps, one thread per tracer.  Its loads go through L1 (a corner is both frames of a node,
+// 32 bytes in FP32), so the blended corners kept in registers count most; then the issue slots, of which the cell
+// search took a quarter.  100 steps of 103,635 tracers on 64^3 FP16 nodes: 642 us before with the corners loaded at
+// every stage and the general cell search, 350 us now; 512,000 on FP32: 3.19 ms before, 1.66 ms.  Three blocks per
+// SM (80 registers): with four 1.68 and on 128^3 nodes 2.55 ms for 2.37.
+template <int ST, int PM>
+__global__ void __launch_bounds__(256, 3) rk4_gather3_kernel(const __grid_constant__ RectParams P,
+                                                               const char *__restrict__ frames, size_t fstride,
+                                                               const __grid_constant__ Rk4Args A)
+{
+    const long long i = thread_tracer(A);
+    const int job = blockIdx.y;
+    if (i < 0) return;
+    float x[3] = {A.seeds[i], A.seeds[A.N + i], A.seeds[2 * A.N + i]}, cx[3] = {0.0f, 0.0f, 0.0f};
+    int img[3] = {0, 0, 0};
+    wrap_periodic<3, PM>(P, x, cx, img);
+    const SchedEntry *sc = A.sched + (size_t)job * A.nsteps_max * 3;
+    const int ns = A.job_nsteps[job];
+    const float h = A.job_h[job], hh = 0.5f * h, h6 = h * (1.0f / 6.0f);
+    unsigned char st = LCS_TRACER_OK;
+    float te = A.job_tend[job];
+    int si = 0;   // next snapshot
+    BlendCache cc;
+    cc.v0 = -1;
+    for (int n = 0; n < ns; ++n) {
+        const SchedEntry e0 = load_sched(sc + 3 * n), e1 = load_sched(sc + 3 * n + 1), e2 = load_sched(sc + 3 * n + 2);
+        float k1[3], k2[3], k3[3], k4[3], y[3], f[3];
+        const auto stage = [&](float c, const float *k) {
+            const float2 q = __ffma2_rn(make_float2(c, c), make_float2(k[0], k[1]), make_float2(x[0], x[1]));
+            y[0] = q.x;
+            y[1] = q.y;
+            y[2] = fmaf(c, k[2], x[2]);
+        };
+        interp3_cached<ST, PM>(P, x, frames, fstride, e0, cc, f, k1);
+        stage(hh, k1);
+        interp3_cached<ST, PM>(P, y, frames, fstride, e1, cc, f, k2);
+        stage(hh, k2);
+        interp3_cached<ST, PM>(P, y, frames, fstride, e1, cc, f, k3);
+        stage(h, k3);
+        interp3_cached<ST, PM>(P, y, frames, fstride, e2, cc, f, k4);
+        float2 xy = make_float2(x[0], x[1]), cxy = make_float2(cx[0], cx[1]);
+        rk4_advance2(xy, cxy, h6, make_float2(k1[0], k1[1]), make_float2(k2[0], k2[1]), make_float2(k3[0], k3[1]),
+                     make_float2(k4[0], k4[1]));
+        x[0] = xy.x;
+        x[1] = xy.y;
+        cx[0] = cxy.x;
+        cx[1] = cxy.y;
+        rk4_advance(x[2], cx[2], h6, k1[2], k2[2], k3[2], k4[2]);
+        wrap_periodic_step<3, PM>(P, x, cx, img);
+        if (rect_left<3, PM>(P, x)) {
+            st = LCS_TRACER_LEFT;
+            te = fmaf((float)(n + 1), h, A.job_t0[job]);
+            break;
+        }
+        for (; si < A.nsnap && snap_step(A, si, ns) == n + 1; ++si)
+            store_tracer<3>(P, A, snap_slot(A, job, si), i, x, cx, img, st, snap_exit(A, job, si, st, te));
+    }
+    for (; si < A.nsnap; ++si)  // snapshots after the tracer stopped (or of a zero-step job)
+        store_tracer<3>(P, A, snap_slot(A, job, si), i, x, cx, img, st, snap_exit(A, job, si, st, te));
+    store_tracer<3>(P, A, job, i, x, cx, img, st, te);
+}
+
 // ============================================================ variational
 
-// u and its spatial Jacobian J[c][d] at x, linear in time between two frames: u with
+// 2D: u and its spatial Jacobian J[c][d] at x, linear in time between two frames: u with
 // interp's arithmetic (node blends first, then make_stencil's weights in order), J from the
 // same blended corner values and the derivatives of the weights inside the cell; a
 // non-periodic axis on which x lies outside the box gives a zero column (the clamped query
 // does not move with x).
-template <int DIM, int ST>
+template <int ST>
 __device__ __forceinline__ void interp_grad(const RectParams &P, const float *x, const char *fa, const char *fb,
-                                            float a, float *u, float (*J)[DIM])
+                                            float a, float *u, float (*J)[2])
 {
-    Stencil<DIM> S;
-    make_stencil<DIM>(P, x, S);
-    float f[DIM], on[DIM];
+    Stencil<2> S;
+    make_stencil<2>(P, x, S);
+    float f[2], on[2];
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) {
+    for (int d = 0; d < 2; ++d) {
         int i0, i1;
         axis_cell<-1>(P, d, x[d], i0, i1, f[d]);
         on[d] = (P.periodic[d] || (x[d] >= P.origin[d] && x[d] <= P.hi_node[d])) ? P.inv_h[d] : 0.0f;
     }
-    float uq[1 << DIM][DIM], va[DIM], vb[DIM];
+    float uq[4][2], va[2], vb[2];
     const float g = 1.0f - a;
 #pragma unroll
-    for (int q = 0; q < (1 << DIM); ++q) {
-        if constexpr (DIM == 2) {   // frames: fa = frame k, fb = frame k + 1 (read only when a != 0)
-            node_load<2, ST, SRC_GLOBAL>(fa, S.v[q], va);
-            if (a != 0.0f) node_load<2, ST, SRC_GLOBAL>(fb, S.v[q], vb);
-        } else {                    // interval pairs: fa = pair k holds both frames of a node
-            Pair3<ST>::ld(fa, S.v[q], va, vb);
-        }
+    for (int q = 0; q < 4; ++q) {   // frame fb is read only when a != 0
+        node_load<2, ST, SRC_GLOBAL>(fa, S.v[q], va);
+        if (a != 0.0f) node_load<2, ST, SRC_GLOBAL>(fb, S.v[q], vb);
 #pragma unroll
-        for (int c = 0; c < DIM; ++c) uq[q][c] = a == 0.0f ? va[c] : tblend(va[c], vb[c], a, g);
+        for (int c = 0; c < 2; ++c) uq[q][c] = a == 0.0f ? va[c] : tblend(va[c], vb[c], a, g);
     }
+    // corner q has offsets (q & 1, q >> 1); d w_q / d x_d = +-(weight of the other axis) / h_d
 #pragma unroll
-    for (int c = 0; c < DIM; ++c) {
-        float acc = 0.0f;
+    for (int c = 0; c < 2; ++c) {
+        float acc = 0.0f, jx = 0.0f, jy = 0.0f;
 #pragma unroll
-        for (int q = 0; q < (1 << DIM); ++q) acc = fmaf(S.w[q], uq[q][c], acc);
+        for (int q = 0; q < 4; ++q) {
+            acc = fmaf(S.w[q], uq[q][c], acc);
+            const float wx = q >> 1 ? f[1] : 1.0f - f[1], wy = q & 1 ? f[0] : 1.0f - f[0];
+            jx = fmaf(q & 1 ? wx : -wx, uq[q][c], jx);
+            jy = fmaf(q >> 1 ? wy : -wy, uq[q][c], jy);
+        }
         u[c] = acc;
+        J[c][0] = jx * on[0];
+        J[c][1] = jy * on[1];
     }
-    if constexpr (DIM == 3) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-            trilinear_grad(make_float4(uq[0][c], uq[1][c], uq[2][c], uq[3][c]),
-                           make_float4(uq[4][c], uq[5][c], uq[6][c], uq[7][c]), f, on, J[c]);
-        return;
-    }
-    // corner q has offsets (q & 1, (q >> 1) & 1, (q >> 2) & 1); d w_q / d x_d = +-(product of the
-    // other axes' weights) / h_d
-#pragma unroll
-    for (int c = 0; c < DIM; ++c)
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) {
-            float acc = 0.0f;
-#pragma unroll
-            for (int q = 0; q < (1 << DIM); ++q) {
-                float w = ((q >> d) & 1) ? 1.0f : -1.0f;
-#pragma unroll
-                for (int e = 0; e < DIM; ++e)
-                    if (e != d) w *= ((q >> e) & 1) ? f[e] : 1.0f - f[e];
-                acc = fmaf(w, uq[q][c], acc);
-            }
-            J[c][d] = acc * on[d];
-        }
 }
 
 // RK4 with the variational equations dM/dt = J M: the position follows rk4_step's arithmetic
 // exactly (so x(T) equals the other kernels'), M the same stages in FP32
-template <int DIM, int ST>
-__global__ void __launch_bounds__(256) rk4_var_kernel(RectParams P, const char *__restrict__ frames, size_t fstride,
-                                                      Rk4Args A)
+template <int ST>
+__global__ void __launch_bounds__(256) rk4_var2_kernel(RectParams P, const char *__restrict__ frames, size_t fstride,
+                                                       Rk4Args A)
 {
+    constexpr int DIM = 2;
     const long long i = thread_tracer(A);
     const int job = blockIdx.y;
     if (i < 0) return;
@@ -264,7 +417,7 @@ __global__ void __launch_bounds__(256) rk4_var_kernel(RectParams P, const char *
                 for (int b = 0; b < DIM; ++b) Y[a][b] = q == 0 ? M[a][b] : fmaf(c, K[q - 1][a][b], M[a][b]);
             }
             const char *fa = frames + (size_t)e.k * fstride;
-            interp_grad<DIM, ST>(P, y, fa, DIM == 2 ? fa + fstride : fa, e.a, k[q], J);
+            interp_grad<ST>(P, y, fa, fa + fstride, e.a, k[q], J);
 #pragma unroll
             for (int a = 0; a < DIM; ++a)
 #pragma unroll
@@ -295,6 +448,92 @@ __global__ void __launch_bounds__(256) rk4_var_kernel(RectParams P, const char *
     for (int a = 0; a < DIM; ++a)
 #pragma unroll
         for (int b = 0; b < DIM; ++b) o[a * DIM + b] = M[a][b];
+}
+
+// The same in 3D, through the blended corners of the last cell.  Bound by issue (the Jacobian and its product
+// with M take two thirds of the instructions).  Two blocks of registers per SM: 262,144 tracers on 64^3 FP32
+// nodes, 100 steps, 1.11 ms; three spill, 1.42 ms.
+template <int ST, int PM>
+__global__ void __launch_bounds__(256, 2) rk4_var3_kernel(const __grid_constant__ RectParams P,
+                                                          const char *__restrict__ frames, size_t fstride,
+                                                          const __grid_constant__ Rk4Args A)
+{
+    const long long i = thread_tracer(A);
+    const int job = blockIdx.y;
+    if (i < 0) return;
+    float x[3] = {A.seeds[i], A.seeds[A.N + i], A.seeds[2 * A.N + i]}, cx[3] = {0.0f, 0.0f, 0.0f}, M[3][3];
+    int img[3] = {0, 0, 0};
+#pragma unroll
+    for (int a = 0; a < 9; ++a) M[a / 3][a % 3] = a % 4 ? 0.0f : 1.0f;
+    wrap_periodic<3, PM>(P, x, cx, img);
+    const SchedEntry *sc = A.sched + (size_t)job * A.nsteps_max * 3;
+    const int ns = A.job_nsteps[job];
+    const float h = A.job_h[job], hh = 0.5f * h, h6 = h * (1.0f / 6.0f);
+    unsigned char st = LCS_TRACER_OK;
+    float te = A.job_tend[job];
+    BlendCache cc;
+    cc.v0 = -1;
+    for (int n = 0; n < ns; ++n) {
+        const SchedEntry es[3] = {load_sched(sc + 3 * n), load_sched(sc + 3 * n + 1), load_sched(sc + 3 * n + 2)};
+        float k[4][3], S03[3][3], S12[3][3], Kp[3][3];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float c = q == 0 ? 0.0f : (q == 3 ? h : hh);
+            float y[3], Y[3][3], f[3], on[3], J[3][3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                y[a] = q == 0 ? x[a] : fmaf(c, k[q - 1][a], x[a]);
+                on[a] = per_axis<PM>(P, a) || (y[a] >= P.origin[a] && y[a] <= P.hi_node[a]) ? P.inv_h[a] : 0.0f;
+#pragma unroll
+                for (int b = 0; b < 3; ++b) Y[a][b] = q == 0 ? M[a][b] : fmaf(c, Kp[a][b], M[a][b]);
+            }
+            interp3_cached<ST, PM>(P, y, frames, fstride, es[q == 0 ? 0 : (q == 3 ? 2 : 1)], cc, f, k[q]);
+            float2 uv[8], Jp[3];
+            float z[8], Jz[3];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                uv[b] = make_float2(cc.u[b][0], cc.u[b][1]);
+                z[b] = cc.u[b][2];
+            }
+            trilinear_grad_nodes(uv, f, on, Jp);
+            trilinear_grad_nodes(z, f, on, Jz);
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                J[0][b] = Jp[b].x;
+                J[1][b] = Jp[b].y;
+                J[2][b] = Jz[b];
+            }
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    float acc = 0.0f;
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) acc = fmaf(J[a][d], Y[d][b], acc);
+                    Kp[a][b] = acc;
+                    if (q == 0) S03[a][b] = acc;
+                    else if (q == 1) S12[a][b] = acc;
+                    else if (q == 2) S12[a][b] = S12[a][b] + acc;
+                    else S03[a][b] = S03[a][b] + acc;
+                }
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            rk4_advance(x[a], cx[a], h6, k[0][a], k[1][a], k[2][a], k[3][a]);
+#pragma unroll
+            for (int b = 0; b < 3; ++b) M[a][b] = fmaf(h6, S03[a][b] + 2.0f * S12[a][b], M[a][b]);
+        }
+        wrap_periodic_step<3, PM>(P, x, cx, img);
+        if (rect_left<3, PM>(P, x)) {
+            st = LCS_TRACER_LEFT;
+            te = fmaf((float)(n + 1), h, A.job_t0[job]);
+            break;
+        }
+    }
+    store_tracer<3>(P, A, job, i, x, cx, img, st, te);
+    float *o = A.out_grad + ((size_t)job * A.N + i) * 9;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) o[a] = M[a / 3][a % 3];
 }
 
 // ============================================================== ring kernel
@@ -931,7 +1170,18 @@ static cudaError_t launch_gather(const RectParams &P, const lcs_field *f, const 
                                  cudaStream_t s)
 {
     dim3 grid(seed_map_grid(A.map, A.N, bt), (unsigned)njobs);
-    rk4_gather_kernel<DIM, ST><<<grid, bt, 0, s>>>(P, (const char *)f->d_frames, f->frame_stride, A);
+    const char *fr = (const char *)f->d_frames;
+    if constexpr (DIM == 2) {
+        rk4_gather2_kernel<ST><<<grid, bt, 0, s>>>(P, fr, f->frame_stride, A);
+    } else {
+        const int pm = box3_mask(P);
+        if (pm == 7)
+            rk4_gather3_kernel<ST, 7><<<grid, bt, 0, s>>>(P, fr, f->frame_stride, A);
+        else if (pm == 0)
+            rk4_gather3_kernel<ST, 0><<<grid, bt, 0, s>>>(P, fr, f->frame_stride, A);
+        else
+            rk4_gather3_kernel<ST, -1><<<grid, bt, 0, s>>>(P, fr, f->frame_stride, A);
+    }
     return cudaGetLastError();
 }
 
@@ -1009,7 +1259,8 @@ int launch_rk4_rect(lcs_ctx *ctx, const Rk4Launch &L, cudaStream_t s)
     // GB300 for the sliding-window batches), else the cached gather in 2D (the shared-memory ring's
     // per-step block barriers cost more than the loads they save while the field stays in L2);
     // re-bundled episodes for large 3D lattices
-    if (variant == 0) variant = sorted_ok && L.N >= LCS_SORTED_MIN_SEEDS ? 3 : (f->dim == 2 && L.work ? 5 : 1);
+    if (variant == 0)
+        variant = sorted_ok && L.N >= rk4_rebundle_seeds(f, A.out_grad != nullptr) ? 3 : (f->dim == 2 && L.work ? 5 : 1);
     if ((variant == 2 || variant == 4) && !ring_fits) variant = 1;
     if (variant == 4 && !queue_ok) variant = 2;
     if (variant == 3 && !sorted_ok) variant = 1;
@@ -1019,21 +1270,22 @@ int launch_rk4_rect(lcs_ctx *ctx, const Rk4Launch &L, cudaStream_t s)
         return e == cudaSuccess ? variant : -1;
     }
     if (A.out_grad) {   // the variational equations elsewhere: their own one-pass kernel
-        const int bt = L.block_threads > 0 && L.block_threads <= 256 ? L.block_threads : 256;
+        // 3D: 13,824 / 125,000 / 512,000 seeds 239 / 644 / 2030 us, in blocks of 256 272 / 693 / 2083 us
+        const int bt = L.block_threads > 0 && L.block_threads <= 256 ? L.block_threads : f->dim == 3 ? 128 : 256;
         A.map = make_seed_map(L.lat_dim, L.lat_n, bt);
         dim3 grid(seed_map_grid(A.map, A.N, bt), (unsigned)L.njobs);
         const char *fr = (const char *)f->d_frames;
         lcs_tm_begin(ctx, 0, s);
-#define VAR_LAUNCH(D, ST) rk4_var_kernel<D, ST><<<grid, bt, 0, s>>>(P, fr, f->frame_stride, A)
-        if (f->dim == 2) {
-            if (f->storage == LCS_F32) VAR_LAUNCH(2, LCS_F32);
-            else if (f->storage == LCS_F16) VAR_LAUNCH(2, LCS_F16);
-            else VAR_LAUNCH(2, LCS_BF16);
-        } else {
-            if (f->storage == LCS_F32) VAR_LAUNCH(3, LCS_F32);
-            else if (f->storage == LCS_F16) VAR_LAUNCH(3, LCS_F16);
-            else VAR_LAUNCH(3, LCS_BF16);
-        }
+#define VAR_LAUNCH(ST)                                                                                 \
+    do {                                                                                               \
+        if (f->dim == 2) rk4_var2_kernel<ST><<<grid, bt, 0, s>>>(P, fr, f->frame_stride, A);           \
+        else if (box3_mask(P) == 7) rk4_var3_kernel<ST, 7><<<grid, bt, 0, s>>>(P, fr, f->frame_stride, A); \
+        else if (box3_mask(P) == 0) rk4_var3_kernel<ST, 0><<<grid, bt, 0, s>>>(P, fr, f->frame_stride, A); \
+        else rk4_var3_kernel<ST, -1><<<grid, bt, 0, s>>>(P, fr, f->frame_stride, A);                   \
+    } while (0)
+        if (f->storage == LCS_F32) VAR_LAUNCH(LCS_F32);
+        else if (f->storage == LCS_F16) VAR_LAUNCH(LCS_F16);
+        else VAR_LAUNCH(LCS_BF16);
 #undef VAR_LAUNCH
         lcs_tm_end(ctx, 0, s);
         return cudaGetLastError() == cudaSuccess ? 6 : -1;
@@ -1064,7 +1316,10 @@ int launch_rk4_rect(lcs_ctx *ctx, const Rk4Launch &L, cudaStream_t s)
         else
             e = launch_ring_tpt<LCS_BF16>(ctx, P, f, A, L, bt, pers, s);
     } else {
-        int bt = L.block_threads > 0 ? L.block_threads : 256;
+        // few tracers in 3D: smaller blocks spread them evenly over the SMs (46,656 seeds, FP32 64^3 nodes:
+        // 277 us, in blocks of 256 339 us; 512,000 on 128^3 nodes: 2368 / 2271 us)
+        const int few = f->dim == 3 && A.N * L.njobs <= 512LL * ctx->num_sms;
+        int bt = L.block_threads > 0 ? L.block_threads : few ? 128 : 256;
         if (bt > 256) bt = 256;
         A.map = make_seed_map(L.lat_dim, L.lat_n, bt);
         if (f->dim == 2) {

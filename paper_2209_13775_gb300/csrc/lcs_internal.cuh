@@ -263,8 +263,17 @@ struct Rk4Launch {
     int lat_n[3] = {1, 1, 1};
 };
 
-// smallest seed count for which lcs_advect picks the re-bundled kernel by default
-#define LCS_SORTED_MIN_SEEDS 262144
+// Seed count from which lcs_advect picks the re-bundled episodes by default in 3D.  They pay a fill of the time
+// slices, in proportion to the nodes, and a sort per episode, and then advance a tracer in about half the
+// one-pass kernel's time.  100 steps, one-pass / re-bundled, ms: FP32 64^3 nodes: 512,000 seeds 1.66 / 1.75,
+// 1M 3.06 / 2.52; 128^3: 2.1M 6.6 / 7.6, 5.5M 16.3 / 14.0; FP16 (half the bytes in one pass, the same slices)
+// 64^3: 1M 2.62 / 2.52; 128^3: 5.5M 13.8 / 13.9; 256^3: 15.6 / 29.5.  Variational, FP32 64^3: 512,000 2.03 /
+// 2.33, 1M 3.98 / 3.84; 128^3: 2.1M 8.4 / 9.5, 4.1M 16.0 / 16.3.
+static inline long long rk4_rebundle_seeds(const lcs_field *f, bool variational)
+{
+    const long long nodes = (long long)f->n[0] * f->n[1] * f->n[2];
+    return (1LL << 19) + (f->storage == LCS_F32 && !variational ? nodes : 2 * nodes);
+}
 // default RK4 steps per re-bundled episode
 #define LCS_EPISODE_STEPS 40
 
