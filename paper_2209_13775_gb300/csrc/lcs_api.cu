@@ -234,59 +234,84 @@ __device__ __forceinline__ __nv_bfloat16 to_store<__nv_bfloat16>(float v) { retu
 // paired with itself).
 // Every frame value is read by at least one slab (frame f by slab f, the last one also as the
 // k + 1 side of the last slab), so the pass also flags any non-finite value in *nonfinite.
-template <typename T>
-__global__ void convert_rect_kernel(const float *__restrict__ src, int nframes, int nslabs, long long nodes, int dim,
-                                    int vec, size_t slab_stride, char *__restrict__ dst, int *__restrict__ nonfinite)
+// A thread stores its node in CONVERT_RUN consecutive slabs, so a frame of an interval pair is read 1 + 1 / 4
+// times instead of twice, in one store of the node's components each (slabs are 256-byte aligned, a node's
+// components a power of two).  Bound by the L1 wavefronts of its two-byte stores before, by memory latency now:
+// 16 frames of 64^3 nodes, 3D to FP16, 51.5 us before, 20.5 us now (50 MB read, 63 MB stored).
+#define CONVERT_RUN 4
+template <typename T, int DIM, int VEC>
+__global__ void __launch_bounds__(256) convert_rect_kernel(const float *__restrict__ src, int nframes, int nslabs,
+                                                           long long nodes, size_t slab_stride,
+                                                           char *__restrict__ dst, int *__restrict__ nonfinite)
 {
-    long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (idx >= (long long)nslabs * nodes) return;
-    long long f = idx / nodes, v = idx % nodes;
-    T *o = reinterpret_cast<T *>(dst + (size_t)f * slab_stride) + v * vec;
+    const long long v = blockIdx.x * 256LL + threadIdx.x;
+    if (v >= nodes) return;
+    constexpr bool PAIR = VEC > DIM;
     bool ok = true;
-    if (dim == 2 && vec == 2) {
-        const float *s = src + idx * 2;
-        ok = isfinite(s[0]) && isfinite(s[1]);
-        o[0] = to_store<T>(s[0]);
-        o[1] = to_store<T>(s[1]);
-    } else if (dim == 2) {  // triangle meshes: (u_k, v_k, u_{k+1}, v_{k+1}) per node
-        long long f1 = f + 1 < nframes ? f + 1 : f;
-        const float *a = src + (f * nodes + v) * 2, *b = src + (f1 * nodes + v) * 2;
-        ok = isfinite(a[0]) && isfinite(a[1]) && isfinite(b[0]) && isfinite(b[1]);
-        o[0] = to_store<T>(a[0]);
-        o[1] = to_store<T>(a[1]);
-        o[2] = to_store<T>(b[0]);
-        o[3] = to_store<T>(b[1]);
-    } else {
-        long long f1 = f + 1 < nframes ? f + 1 : f;
-        const float *a = src + (f * nodes + v) * 3, *b = src + (f1 * nodes + v) * 3;
-        for (int c = 0; c < 3; ++c) {
-            ok = ok && isfinite(a[c]) && isfinite(b[c]);
-            o[c] = to_store<T>(a[c]);
-            o[4 + c] = to_store<T>(b[c]);
+    for (long long f0 = (long long)blockIdx.y * CONVERT_RUN; f0 < nslabs; f0 += (long long)gridDim.y * CONVERT_RUN) {
+        float a[DIM], b[DIM];
+        const auto read = [&](long long f, float *r) {
+            const float *s = src + (f * nodes + v) * DIM;
+#pragma unroll
+            for (int c = 0; c < DIM; ++c) {
+                r[c] = __ldg(s + c);
+                ok = ok && isfinite(r[c]);
+            }
+        };
+        read(f0, a);
+#pragma unroll
+        for (int q = 0; q < CONVERT_RUN; ++q) {
+            const long long f = f0 + q;
+            if (f >= nslabs) break;
+            if (PAIR || q + 1 < CONVERT_RUN) {   // the next frame: this slab's other side, the next one's first
+                if (f + 1 < nframes && (PAIR || f + 1 < nslabs)) {
+                    read(f + 1, b);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < DIM; ++c) b[c] = a[c];
+                }
+            }
+            struct alignas(VEC * sizeof(T)) Rec {
+                T t[VEC];
+            } o;
+#pragma unroll
+            for (int c = 0; c < VEC; ++c) o.t[c] = to_store<T>(0.0f);
+#pragma unroll
+            for (int c = 0; c < DIM; ++c) {
+                o.t[c] = to_store<T>(a[c]);
+                if (PAIR) o.t[VEC / 2 + c] = to_store<T>(b[c]);
+                a[c] = b[c];
+            }
+            *reinterpret_cast<Rec *>(dst + (size_t)f * slab_stride + sizeof(Rec) * v) = o;
         }
-        o[3] = to_store<T>(0.0f);
-        o[7] = to_store<T>(0.0f);
     }
     if (!ok) atomicOr(nonfinite, 1);
+}
+
+template <typename T>
+static cudaError_t convert_typed(const float *src, int nframes, int nslabs, long long nodes, int dim, int vec,
+                                 size_t slab_stride, char *dst, int *nonfinite, cudaStream_t s)
+{
+    const int runs = (nslabs + CONVERT_RUN - 1) / CONVERT_RUN;
+    const dim3 grid((unsigned)((nodes + 255) / 256), (unsigned)std::min(runs, 65535));
+    if (dim == 2 && vec == 2)
+        convert_rect_kernel<T, 2, 2><<<grid, 256, 0, s>>>(src, nframes, nslabs, nodes, slab_stride, dst, nonfinite);
+    else if (dim == 2)
+        convert_rect_kernel<T, 2, 4><<<grid, 256, 0, s>>>(src, nframes, nslabs, nodes, slab_stride, dst, nonfinite);
+    else
+        convert_rect_kernel<T, 3, 8><<<grid, 256, 0, s>>>(src, nframes, nslabs, nodes, slab_stride, dst, nonfinite);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_convert_rect(const float *src, int nframes, int nslabs, long long nodes, int dim, int vec,
                                 int storage, size_t slab_stride, void *dst, int *nonfinite, cudaStream_t s)
 {
-    long long total = (long long)nslabs * nodes;
-    if (total == 0) return cudaSuccess;
-    int bt = 256;
-    unsigned grid = (unsigned)((total + bt - 1) / bt);
+    if (nslabs == 0 || nodes == 0) return cudaSuccess;
     if (storage == LCS_F32)
-        convert_rect_kernel<float>
-            <<<grid, bt, 0, s>>>(src, nframes, nslabs, nodes, dim, vec, slab_stride, (char *)dst, nonfinite);
-    else if (storage == LCS_F16)
-        convert_rect_kernel<__half>
-            <<<grid, bt, 0, s>>>(src, nframes, nslabs, nodes, dim, vec, slab_stride, (char *)dst, nonfinite);
-    else
-        convert_rect_kernel<__nv_bfloat16>
-            <<<grid, bt, 0, s>>>(src, nframes, nslabs, nodes, dim, vec, slab_stride, (char *)dst, nonfinite);
-    return cudaGetLastError();
+        return convert_typed<float>(src, nframes, nslabs, nodes, dim, vec, slab_stride, (char *)dst, nonfinite, s);
+    if (storage == LCS_F16)
+        return convert_typed<__half>(src, nframes, nslabs, nodes, dim, vec, slab_stride, (char *)dst, nonfinite, s);
+    return convert_typed<__nv_bfloat16>(src, nframes, nslabs, nodes, dim, vec, slab_stride, (char *)dst, nonfinite, s);
 }
 
 static lcs_status upload_frames(lcs_ctx *ctx, lcs_field *f, const float *frames, int on_device)
