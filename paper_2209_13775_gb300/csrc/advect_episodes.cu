@@ -273,21 +273,21 @@ __global__ void ep_slice_table_kernel(const SchedEntry *__restrict__ sched, int 
 // Time slices.  Slice j is the field blended to stage time stab[j] in FP32 (interp3p's
 // arithmetic on the stored frames, widened from FP16/BF16 storage), as xy-quads on a lattice extended by
 // a halo of SLICE_HALO nodes on each side of every periodic axis: extended node (I, J, K) holds,
-// for c = 0, 1, 2 in turn, the float4 (u_c(i, j, k), u_c(i1, j, k), u_c(i, j1, k), u_c(i1, j1, k))
+// for c = 0, 1, 2, the float4 (u_c(i, j, k), u_c(i1, j, k), u_c(i, j1, k), u_c(i1, j1, k))
 // with (i, j, k) the field node the extended node wraps to and i1, j1 the next node along
-// x and y (wrapped, or clamped on a closed axis).  A trilinear stencil is then two 16-byte
-// loads per component (its two z-rows), the three of a row in one 48-byte run (interleaving
-// the components rather than keeping three planes cut the episode kernel from 113.2 to
-// 111.2 ms per 400 steps at C2), and stencil points a few cells outside the periodic box need
-// no index wrapping: the halo holds the wrapped values.
+// x and y (wrapped, or clamped on a closed axis).  The quads of u and v stand side by side in one
+// 32-byte record, those of w in a plane behind them, so a trilinear stencil is a 32-byte and a 16-byte
+// load for each of its two z-rows.  The L1 data stage bounds the advection: three 16-byte loads a row,
+// the quads of a node in one 48-byte run, kept it 94% busy (10.35 ms per 40 steps at 16.8M tracers on
+// 128^3 nodes, 400 steps 126.0 ms with the slices); the 32-byte loads take a fifth off its wavefronts (80% busy, 10.08 ms,
+// 124.4 ms), and the loads' latency at half the warps of an SM bounds what is left.  Stencil
+// points a few cells outside the periodic box need no index wrapping: the halo holds the wrapped values.
 //
 // Rows and planes of a slice are padded (pitches R and Q nodes, R = 4 and Q = 2 mod 8) so that
-// the 8 nodes of any 2 x 2 x 2 block of cells start in 8 different 16-byte bank groups of a
-// 128-byte line: the L1 data stage serves the 8 lanes of a quarter warp in one wavefront only
-// when no two of them read different addresses in the same bank group, and the stencil loads of
-// nearby tracers then rarely collide.  Unpadded, z-neighbours (Q = 132^2 = 0 mod 8 on the ABC
-// grid) always collided; a count of the collisions along RK4 trajectories of the ABC flow gave
-// 1.78 wavefronts per quarter warp unpadded, 1.01 padded.
+// lanes in neighbouring cells rarely read different addresses in the same banks of the L1 data
+// stage, which would take a wavefront each: z-neighbours always collide unpadded (Q = 132^2 = 0 mod 8
+// on the ABC grid).  The same advection with R, Q mod 8 = 4, 2 (or 4, 6) 124.4 ms; 4, 3: 125.9; 4, 1:
+// 126.1; 5, 2: 126.5; 6, 3: 128.0; 1, 2: 131.9; 2, 1: 132.7; 2, 4: 133.1; 3, 2: 133.5; 0, 0: 135.9.
 #define SLICE_HALO 2
 
 struct SliceGeom {
@@ -296,7 +296,10 @@ struct SliceGeom {
     int R;           // row pitch in nodes (>= N[0], = 4 mod 8)
     long long nxy;   // plane pitch in nodes (>= R * N[1], = 2 mod 8)
     long long nodes; // nodes of one slice plane, padding included (nxy * N[2])
+    unsigned wofs;   // float4 from a slice's (u, v) quads to its w quads
 };
+
+static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 static SliceGeom slice_geom(const lcs_field *f)
 {
@@ -309,6 +312,7 @@ static SliceGeom slice_geom(const lcs_field *f)
     const long long q = (long long)G.R * G.N[1];
     G.nxy = q + ((2 - q) & 7);
     G.nodes = G.nxy * G.N[2];
+    G.wofs = (unsigned)(2 * (al256(16 * (size_t)G.nodes) / 16));   // (nodes <= 2^30)
     return G;
 }
 
@@ -329,8 +333,8 @@ __global__ void ep_slice_fill_kernel(RectParams P, SliceGeom G, const char *__re
                                      const SchedEntry *__restrict__ stab, const int *__restrict__ nsl,
                                      float4 *__restrict__ slices, size_t plane_stride)
 {
-    // a block's 256 nodes are consecutive, so their interleaved quads (3 per node) form one run
-    // of 768 float4 per slice: staged in shared memory and stored coalesced (padding nodes get 0)
+    // a block's 256 nodes are consecutive, so their quads form two runs per slice, 512 float4 of (u, v) and
+    // 256 of w: staged in shared memory and stored coalesced (padding nodes get 0)
     __shared__ float4 stage[256 * 3];
     const long long vb = (long long)blockIdx.x * 256;
     const long long v = vb + threadIdx.x;
@@ -375,21 +379,22 @@ __global__ void ep_slice_fill_kernel(RectParams P, SliceGeom G, const char *__re
                 float u[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) u[q] = e.a == 0.0f ? ua[q][c] : tblend(ua[q][c], ub[q][c], e.a, g);
-                stage[3 * threadIdx.x + c] = make_float4(u[0], u[1], u[2], u[3]);
+                stage[c < 2 ? 2 * threadIdx.x + c : 512 + threadIdx.x] = make_float4(u[0], u[1], u[2], u[3]);
             }
         } else {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) stage[3 * threadIdx.x + c] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (int c = 0; c < 3; ++c) stage[c < 2 ? 2 * threadIdx.x + c : 512 + threadIdx.x] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
         __syncthreads();
-        float4 *base = slices + (size_t)j * 3 * plane_stride + 3 * vb;
-        for (int q = threadIdx.x; q < 3 * nb; q += 256) base[q] = stage[q];
+        float4 *base = slices + (size_t)j * 3 * plane_stride + 2 * vb, *wb = base - vb + G.wofs;
+        for (int q = threadIdx.x; q < 2 * nb; q += 256) base[q] = stage[q];
+        if (threadIdx.x < nb) wb[threadIdx.x] = stage[512 + threadIdx.x];
         __syncthreads();
     }
 }
 
 // The second layout: plain nodes (u, v, w, 0), the field blended to the slice's time and nothing repeated.  A
-// stencil is eight 16-byte loads for the quads' six, a slice a third of the bytes to write: for lattices
+// stencil is eight 16-byte loads for the quads' two of 16 and two of 32, a slice a third of the bytes to write: for lattices
 // with few tracers per node, where writing the slices costs as much as reading them (slices_plain).  Two
 // x-neighbours in one 32-byte record (four loads, 32 bytes to write) was slower than nodes on sparse
 // lattices and than quads on dense ones (132.4 ms): at eight tracers per node every layout keeps the L1
@@ -558,6 +563,13 @@ struct CornerCache {
     }
 };
 
+__device__ __forceinline__ void ldg_quads(const float4 *p, float4 &a, float4 &b)
+{
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(p));
+}
+
 // u(x) from slice `slice` at pl; the products and their order are interp3p's: corners (i0,j0,k0),
 // (i1,j0,k0), (i0,j1,k0), (i1,j1,k0), then k1.
 template <int LAY>
@@ -569,8 +581,8 @@ __device__ __forceinline__ void interp3q(int v0, const float *w, const float4 *_
         for (int r = 0; r < 2; ++r) {
             const int v = v0 + r * (int)G.nxy;
             if constexpr (LAY == QUAD) {
-#pragma unroll
-                for (int c = 0; c < 3; ++c) cc.q[3 * r + c] = __ldg(pl + 3 * v + c);
+                ldg_quads(pl + 2 * v, cc.q[3 * r], cc.q[3 * r + 1]);
+                cc.q[3 * r + 2] = __ldg(pl + G.wofs + v);
             } else {
                 cc.q[4 * r] = __ldg(pl + v);
                 cc.q[4 * r + 1] = __ldg(pl + v + 1);
@@ -851,7 +863,6 @@ __global__ void ep_finalize_kernel(RectParams P, const Tracer *__restrict__ S, R
 
 // ------------------------------------------------------------------- driver
 
-static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // coarsen cell keys so that at most 2^24 bins exist (the scan handles 4096 tiles of 4096)
 static int sort_shift(long long nodes)
@@ -863,7 +874,7 @@ static int sort_shift(long long nodes)
 
 // Plain nodes rather than quads in the slices: wherever the writes saved outweigh the wider gathers.  RK4,
 // 100 steps on 128^3 nodes, quads / nodes: 0.12 tracers per node 5.86 / 2.99 ms, 1: 9.24 / 7.36, 2: 12.8 /
-// 11.6, 4: 19.5 / 18.8, 8 (400 steps): 129.1 / 131.1.  The variational kernel, bound by issue, gains at any
+// 11.6, 4: 19.5 / 18.8, 8 (400 steps): 127.5 / 131.1.  The variational kernel, bound by issue, gains at any
 // density: 1 per node 12.07 / 9.58 ms, 2: 18.95 / 16.4.
 static bool slices_plain(const lcs_field *f, long long N, bool var) { return var || N < 6 * f->nodes; }
 
