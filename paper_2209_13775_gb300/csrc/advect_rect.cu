@@ -1258,9 +1258,8 @@ int launch_rk4_rect(lcs_ctx *ctx, const Rk4Launch &L, cudaStream_t s)
     // default: 2D time slices when lcs_advect reserved them (at most 2 GiB; the autotuner's choice on
     // GB300 for the sliding-window batches), else the cached gather in 2D (the shared-memory ring's
     // per-step block barriers cost more than the loads they save while the field stays in L2);
-    // re-bundled episodes for large 3D lattices
-    if (variant == 0)
-        variant = sorted_ok && L.N >= rk4_rebundle_seeds(f, A.out_grad != nullptr) ? 3 : (f->dim == 2 && L.work ? 5 : 1);
+    // re-bundled episodes for large 3D lattices (lcs_advect reserves their memory from rk4_rebundle_seeds on)
+    if (variant == 0) variant = sorted_ok ? 3 : (f->dim == 2 && L.work ? 5 : 1);
     if ((variant == 2 || variant == 4) && !ring_fits) variant = 1;
     if (variant == 4 && !queue_ok) variant = 2;
     if (variant == 3 && !sorted_ok) variant = 1;

@@ -789,7 +789,8 @@ static AdvectLayout advect_layout(const lcs_field *f, const lcs_seeds *s, const 
             align256(sizeof(int) * LCS_MAX_SNAP) + align256(sizeof(float) * J.njobs * LCS_MAX_SNAP);
     Ly.sb = align256(sizeof(SchedEntry) * 3 * (size_t)J.njobs * std::max(J.nsteps_max, 1));
     Ly.want_work = f->dim == 3 &&
-                   (o->variant == 3 || (o->variant == 0 && s->N >= rk4_rebundle_seeds(f, o->variational != 0)));
+                   (o->variant == 3 ||
+                    (o->variant == 0 && s->N >= rk4_rebundle_seeds(f, o->variational != 0, J.nsteps_max)));
     Ly.E = o->episode_steps > 0 ? std::min(o->episode_steps, 1024) : LCS_EPISODE_STEPS;
     Ly.wb = Ly.want_work ? rk4_sorted_scratch_bytes(s->N, f, Ly.E, o->variational != 0) : 0;
     if (f->dim == 2 && f->kind == LCS_RECTILINEAR && (o->variant == 5 || o->variant == 0)) {

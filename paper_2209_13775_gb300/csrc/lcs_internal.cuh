@@ -265,15 +265,24 @@ struct Rk4Launch {
 
 // Seed count from which lcs_advect picks the re-bundled episodes by default in 3D.  They pay a fill of the time
 // slices, in proportion to the nodes, and a sort per episode, and then advance a tracer in about half the
-// one-pass kernel's time.  100 steps, one-pass / re-bundled, ms: FP32 64^3 nodes: 512,000 seeds 1.66 / 1.75,
-// 1M 3.06 / 2.52; 128^3: 2.1M 6.6 / 7.6, 5.5M 16.3 / 14.0; FP16 (half the bytes in one pass, the same slices)
-// 64^3: 1M 2.62 / 2.52; 128^3: 5.5M 13.8 / 13.9; 256^3: 15.6 / 29.5.  Variational, FP32 64^3: 512,000 2.03 /
-// 2.33, 1M 3.98 / 3.84; 128^3: 2.1M 8.4 / 9.5, 4.1M 16.0 / 16.3.
-static inline long long rk4_rebundle_seeds(const lcs_field *f, bool variational)
+// one-pass kernel's time, or less the farther the lattice has been carried apart (steps: of the longest job).
+// ABC flow, one-pass / re-bundled, ms:
+//   FP32, 100 steps of 0.02: 64^3 nodes: 512,000 seeds 1.66 / 1.75, 1M 3.06 / 2.52; 128^3: 2.1M 6.6 / 7.6, 5.5M
+//     16.3 / 14.0; 400 steps: 64^3: 262,144 5.9 / 4.9; 128^3: 262,144 6.7 / 13.2, 1M 20.4 / 19.6, 2.1M 39.0 / 30.1
+//   FP16 (half the bytes in one pass, the same slices), 100 steps: 64^3: 1M 2.62 / 2.52; 128^3: 5.5M 13.8 / 13.9;
+//     400 steps: 64^3: 512,000 6.3 / 6.9, 778,688 9.6 / 8.5; 128^3: 2.1M 28.3 / 29.8, 2.7M 37.4 / 35.7
+//   variational (bound by issue), FP32, 100 steps: 64^3: 512,000 2.03 / 2.33, 1M 3.98 / 3.84; 128^3: 2.1M
+//     8.4 / 9.5, 4.1M 16.0 / 16.3; 400 steps: 64^3: 262,144 5.4 / 5.8, 512,000 9.6 / 9.1; 128^3: 1M 21.9 / 22.2
+static inline long long rk4_rebundle_seeds(const lcs_field *f, bool variational, int steps)
 {
     const long long nodes = (long long)f->n[0] * f->n[1] * f->n[2];
-    return (1LL << 19) + (f->storage == LCS_F32 && !variational ? nodes : 2 * nodes);
+    const bool half = f->storage != LCS_F32 && !variational;
+    const long long at100 = (1LL << 19) + (half || variational ? 2 * nodes : nodes);
+    const int longest = half ? 200 : 300, s = steps < 100 ? 100 : steps > longest ? longest : steps;
+    const long long n = at100 * 100 / s;
+    return n > (1LL << 18) ? n : 1LL << 18;
 }
+
 // default RK4 steps per re-bundled episode
 #define LCS_EPISODE_STEPS 40
 
