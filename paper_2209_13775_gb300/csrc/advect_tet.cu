@@ -240,6 +240,7 @@ __global__ void __launch_bounds__(256) rk4_mesh_var_kernel(MD T, Rk4Args A, cons
 
 // largest k with t_k <= t (after the periodic wrap), clamped to [0, nf-2]; the weight of
 // frame k+1, clamped to [0, 1] unless time is periodic.  times: FP32 copy in shared memory
+template <bool HINT>
 __device__ __forceinline__ void bracket_f32(const float *times, int nf, int tp, float period, float t, int &k,
                                             float &a)
 {
@@ -253,10 +254,10 @@ __device__ __forceinline__ void bracket_f32(const float *times, int nf, int tp, 
     }
     float tt = t;
     if (tp) tt = t - period * floorf((t - times[0]) / period);
-    float t0 = times[k], t1 = times[k + 1];
-    if (!(t0 <= tt && tt < t1)) {
+    float t0 = HINT ? times[k] : 0.0f, t1 = HINT ? times[k + 1] : 0.0f;
+    if (!HINT || !(t0 <= tt && tt < t1)) {
         int lo = 0, hi = nf - 1;
-        if (tt >= t1 && k + 2 < nf && tt < times[k + 2]) {
+        if (HINT && tt >= t1 && k + 2 < nf && tt < times[k + 2]) {
             lo = k + 1;
         } else {
             while (lo < hi) {
@@ -283,12 +284,16 @@ __device__ __forceinline__ void eval_state_init(NoEvalState &) {}
 __device__ __forceinline__ void eval_state_init(TriCache &cc) { tri_cache_init(cc); }
 
 // velocity at (x, t) on a tet mesh; walks from *cell.  Returns TET_INSIDE / OUTSIDE / WALKFAIL
-template <int ST>
+template <int ST, bool FEW>
 struct TetEval {
     static constexpr int DIM = 3;
-    // three blocks (80 registers) on tets: 3.23 against 3.43 ms per pass of four (2.1M seeds, 1M tets).  A
-    // register cache of the last cell (TetCache) costs more here than the few hits of long steps give (3.64)
-    static constexpr int MINB = 3;
+    // Three blocks (80 registers) and the bracket tried first, or four (64, some spills).  Three / four, us: F32, 1M
+    // tets: 57,600 seeds 391 / 429, 204,800 437 / 494, 2.1M 3077 / 3107; 2.4M tets: 2.1M seeds 3529 / 3444; FP16, 1M
+    // tets: 57,600 seeds 395 / 408, 204,800 414 / 440, 480,000 791 / 753, 2.1M 2925 / 2754.  (The bracket tried
+    // first in four F32 blocks spills more: 3260 and 3807.)  A register cache of the last cell (TetCache)
+    // costs more here than the few hits of long steps give (3640).
+    static constexpr int MINB = FEW ? 3 : 4;
+    static constexpr bool HINT = FEW || ST != LCS_F32;
     using State = NoEvalState;
     TetDev T;
     __device__ __forceinline__ int eval(const float *x, int k, float a, int *cell, float *u, State &) const
@@ -305,6 +310,7 @@ template <int ST>
 struct TriEval {
     static constexpr int DIM = 2;
     static constexpr int MINB = 4;
+    static constexpr bool HINT = true;
     using State = TriCache;   // the seven stage points of a step mostly share a cell and an interval
     TriDev T;
     __device__ __forceinline__ int eval(const float *x, int k, float a, int *cell, float *u, State &cc) const
@@ -325,6 +331,7 @@ template <int ST>
 struct Rect2Eval {
     static constexpr int DIM = 2;
     static constexpr int MINB = 4;
+    static constexpr bool HINT = true;
     using State = NoEvalState;
     RectParams P;
     const char *frames;
@@ -343,6 +350,7 @@ template <int ST, bool UNIT>
 struct Rect2BoxEval {
     static constexpr int DIM = 2;
     static constexpr int MINB = 4;
+    static constexpr bool HINT = true;
     using State = NoEvalState;
     Box2 B;
     int nx;
@@ -366,6 +374,7 @@ template <int ST>
 struct Rect3Eval {
     static constexpr int DIM = 3;
     static constexpr int MINB = 4;
+    static constexpr bool HINT = true;
     using State = NoEvalState;
     RectParams P;
     const char *pairs;
@@ -405,7 +414,7 @@ __device__ __forceinline__ int dp_eval(const EV &E, const Dp45Args &A, const flo
                                        int *cell, float *u, typename EV::State &cs, int &k)
 {
     float a;
-    bracket_f32(times, A.nf, A.tp, A.period, t, k, a);
+    bracket_f32<EV::HINT>(times, A.nf, A.tp, A.period, t, k, a);
     return E.eval(x, k, a, cell, u, cs);
 }
 
@@ -647,12 +656,18 @@ cudaError_t launch_dp45(lcs_ctx *ctx, const lcs_field *f, const Dp45Args &A0, in
     } else if (f->kind == LCS_TET) {
         A.rect_left = 0;
         const TetDev T = tet_dev(f, walk_limit);
+        // many tracers on a mesh whose maps and neighbours (80 bytes a cell) lie beyond the L2, or whose frames
+        // take half the bytes: more resident warps pay more than registers do (TetEval)
+        const bool few = A.N * njobs < (1LL << 18) || (f->storage == LCS_F32 && 80 * f->ncells <= (128LL << 20));
         if (f->storage == LCS_F32)
-            e = dp45_go(TetEval<LCS_F32>{T}, A, P, njobs, bt, s);
+            e = few ? dp45_go(TetEval<LCS_F32, true>{T}, A, P, njobs, bt, s)
+                    : dp45_go(TetEval<LCS_F32, false>{T}, A, P, njobs, bt, s);
         else if (f->storage == LCS_F16)
-            e = dp45_go(TetEval<LCS_F16>{T}, A, P, njobs, bt, s);
+            e = few ? dp45_go(TetEval<LCS_F16, true>{T}, A, P, njobs, bt, s)
+                    : dp45_go(TetEval<LCS_F16, false>{T}, A, P, njobs, bt, s);
         else
-            e = dp45_go(TetEval<LCS_BF16>{T}, A, P, njobs, bt, s);
+            e = few ? dp45_go(TetEval<LCS_BF16, true>{T}, A, P, njobs, bt, s)
+                    : dp45_go(TetEval<LCS_BF16, false>{T}, A, P, njobs, bt, s);
     } else if (f->dim == 2) {
         A.rect_left = 1;
         const char *fr = (const char *)f->d_frames;
