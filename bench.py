@@ -440,10 +440,10 @@ def our_arm(args, rank, world, local):
                      "traffic_note": "ncu DRAM bytes per tracer-step of the small case (64^3 field, 128^3 "
                                      "seeds) scaled by this launch's tracer-steps "
                                      "(profiles/ep_advect3_traffic.md)",
-                     "limiter": "the L1 data stage (ncu, small case: 79% of its one-wavefront-per-cycle peak; "
-                                "7.7 wavefronts per 16-byte gather request against 4 when a quarter warp's "
-                                "lanes read at most 4 lines: the re-bundled tracers spread over 5-8 rows of "
-                                "cells within a few steps); issue 69%, 470 instructions per warp-step"},
+                     "limiter": "the gathers (ncu, 40-step launch at this size): the L1 data stage 80% busy, its "
+                                "hit rate 55% (the re-bundled tracers spread over 5-8 rows of cells within a few "
+                                "steps), issue 67%, 403 instructions per warp-step, half the warps of an SM "
+                                "resident (64 registers)"},
         "phases_ms_per_step": {k: v[0] / args.steps for k, v in phase.items()},
         "clocks": clocks,
         "e2e": {"value": world * N / e2e_el if e2e_t else None, "unit": "seeds/s", "h2d_bytes_per_step": h2d,
@@ -646,8 +646,8 @@ def c3_arm(args, rank, world, local):
         "tracer_steps_per_s": tracer_steps * args.steps / el,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                      "frac": achieved / fp32_peak, "traffic": None,
-                     "kernel": {1: "rk4_gather_kernel", 2: "rk4_ring2d_kernel", 4: "rk4_ring2d_kernel (persistent)",
-                                5: "rk4_slice2d_kernel (with slice2d_fill_kernel)"}.get(opts.variant, "?")
+                     "kernel": {1: "rk4_gather2_kernel", 2: "rk4_ring2d_kernel", 4: "rk4_ring2d_kernel (persistent)",
+                                5: "rk4_slice2d_box_kernel (with slice2d_fill_kernel)"}.get(opts.variant, "?")
                                + " (variant %d)" % opts.variant, "flop_per_launch": flops,
                      "avg_launch_ms": adv_ms / max(adv_n, 1), "launches": adv_n,
                      "peak_basis": "152 SMs x 128 FP32 lanes x 2 x %.0f MHz (%s sm_max_mhz)" % (sm_mhz, pk_kind)},

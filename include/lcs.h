@@ -265,7 +265,9 @@ typedef struct {
                                        items longest-job first (2D, batches);
                                    5 = the field blended once to every stage time of
                                        every job (2D time slices; up to 16 GiB; the
-                                       default in 2D when they take at most 2 GiB)     */
+                                       default in 2D when they take at most 2 GiB).
+                                   The default in 3D is 1, and 3 from about as many
+                                   tracers as the field has nodes on (262144 at least) */
     const void *surrogate;      /* LCS_SURROGATE: the lcs_mlp to step with            */
     int episode_steps;          /* variant 3: RK4 steps between re-bundlings (0 = 40) */
     int tracers_per_thread;     /* variants 2 and 4: 1 or 2 tracers per thread (0 = 1) */
@@ -456,7 +458,8 @@ lcs_status lcs_cauchy_green(lcs_ctx *ctx, const lcs_flowmap *fm, int job, double
                             int on_device);
 
 /* FTLE sigma = ln(sqrt(lambda_max(C))) / |T| (Sec. 1: the FTLE is derived from
- * the largest eigenvalue of C) as FP32 [N], NaN where C is undefined;
+ * the largest eigenvalue of C) as FP32 [N], NaN where C is undefined, computed
+ * with 46-bit arithmetic from the FP32 positions whatever else is asked for;
  * optionally lambda_max [N] FP64 and C (as lcs_cauchy_green) from the same
  * pass.  lambda_max and C may be NULL.  job = -1 writes every job.
  * Errors: as lcs_cauchy_green.                                              */
@@ -492,8 +495,9 @@ lcs_status lcs_ftle_early(lcs_ctx *ctx, const lcs_field *field, const lcs_seeds 
  * both among the filter's per-seed outputs), C as lcs_cauchy_green.  eigval [N][dim] FP64 in
  * ascending order; eigvec [N][dim][dim] FP64, eigvec[(p*dim + k)*dim + r]
  * = component r of the unit eigenvector of eigval[p][k], its largest-magnitude
- * component positive.  Cyclic Jacobi rotations in FP64 to a relative
- * off-diagonal threshold (16 sweeps at most).  NaN where C is undefined.
+ * component positive.  2x2, and 3x3 whose split solution (a double-FP32 root,
+ * corrected in FP64) does not settle: cyclic Jacobi rotations in FP64 to a
+ * relative off-diagonal threshold (16 sweeps at most).  NaN where C is undefined.
  * Either output may be NULL; job = -1 writes every job.
  * Errors: LCS_EINVAL, LCS_ECUDA.                                            */
 lcs_status lcs_cg_eigen(lcs_ctx *ctx, const lcs_flowmap *fm, int job, double *eigval, double *eigvec,

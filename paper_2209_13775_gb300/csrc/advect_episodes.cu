@@ -17,8 +17,8 @@
 //
 // Per episode the field is blended once, in FP32, to every distinct stage time of the
 // episode (a "time slice", on a lattice with a halo on periodic axes; stored as xy-quads of the three
-// components interleaved per node, or as plain nodes where tracers are few); the advection then reads
-// six or eight 16-byte words per stencil, and keeps the last stencil's corners in registers for the next
+// components, or as plain nodes where tracers are few); the advection then reads two 32-byte and two
+// 16-byte words, or eight 16-byte words, per stencil, and keeps the last stencil's corners in registers for the next
 // stage that reads the same slice from the same cell.  FP16/BF16 storage is widened in the fill.
 #include "rect_device.cuh"
 
@@ -279,9 +279,10 @@ __global__ void ep_slice_table_kernel(const SchedEntry *__restrict__ sched, int 
 // 32-byte record, those of w in a plane behind them, so a trilinear stencil is a 32-byte and a 16-byte
 // load for each of its two z-rows.  The L1 data stage bounds the advection: three 16-byte loads a row,
 // the quads of a node in one 48-byte run, kept it 94% busy (10.35 ms per 40 steps at 16.8M tracers on
-// 128^3 nodes, 400 steps 126.0 ms with the slices); the 32-byte loads take a fifth off its wavefronts (80% busy, 10.08 ms,
-// 124.4 ms), and the loads' latency at half the warps of an SM bounds what is left.  Stencil
-// points a few cells outside the periodic box need no index wrapping: the halo holds the wrapped values.
+// 128^3 nodes, 400 steps 126.0 ms with the slices); the 32-byte loads take a fifth off its wavefronts
+// (80% busy, 10.08 ms, 124.4 ms), and the loads' latency at half the warps of an SM bounds what is left.
+// Stencil points a few cells outside the periodic box need no index wrapping: the halo holds the wrapped
+// values.
 //
 // Rows and planes of a slice are padded (pitches R and Q nodes, R = 4 and Q = 2 mod 8) so that
 // lanes in neighbouring cells rarely read different addresses in the same banks of the L1 data

@@ -10,8 +10,9 @@
 // four fused stage evaluations.  All tracers of a launch share the time
 // schedule, so the frame bracket (k, alpha) of every stage is computed once
 // per (job, step, stage) in FP64 by a small kernel and read as a warp-uniform
-// broadcast.  Two kernels:
-//   * gather: nodes read through L1/L2 (any field size, 2D and 3D);
+// broadcast.  Three families of kernels:
+//   * gather: nodes read through L1/L2 (any field size, 2D and 3D; in 3D the last cell's corners kept);
+//   * 2D time slices: the field blended once to every stage time;
 //   * ring (2D): a block keeps three whole frames in shared memory, staged by
 //     bulk asynchronous copies (cp.async.bulk + mbarrier) and prefetched one
 //     step ahead, so the stage evaluations read shared memory only.
