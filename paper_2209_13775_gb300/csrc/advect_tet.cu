@@ -568,7 +568,13 @@ cudaError_t launch_rk4_tet(lcs_ctx *ctx, const Rk4Launch &L, const int *cells0, 
     A.out_grad = L.out_grad;
     if (L.N == 0) return cudaSuccess;
     const int bt = L.block_threads > 0 && L.block_threads <= 256 ? L.block_threads : 128;
-    A.map = make_seed_map(L.lat_dim, L.lat_n, bt);
+    // Warps take tiles of the lattice (triangles: 4.2M seeds 31.7 -> 28.3 ms; 16,384: 3.11 -> 3.03; tets: 64 x 64 x 512
+    // seeds 6.33 -> 5.86 ms), but rows of it on triangles for a few warps, as slow as their slowest lane (2048
+    // seeds 2.18 ms, in tiles 2.25), and on tets where the tiles at the lattice's edges would leave more than a
+    // sixteenth of the lanes idle (45 x 45 x 301 seeds 1.66 ms, in tiles 1.73)
+    A.map = make_seed_map(f->kind == LCS_TRI && L.N * L.njobs < 8192 ? 0 : L.lat_dim, L.lat_n, bt);
+    if (f->kind == LCS_TET && (long long)seed_map_grid(A.map, L.N, bt) * bt > L.N + L.N / 16 + bt)
+        A.map = make_seed_map(0, L.lat_n, bt);
     dim3 grid(seed_map_grid(A.map, L.N, bt), (unsigned)L.njobs);
     if (A.out_grad) {   // the variational equations
         lcs_tm_begin(ctx, 0, s);
