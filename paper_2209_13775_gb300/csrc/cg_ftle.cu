@@ -14,7 +14,7 @@
 //    scaled matrix (Smith 1961), whose trigonometric root is taken in FP32 and polished by two FP64
 //    Newton steps, and by Jacobi rotations where the two largest eigenvalues (nearly) coincide.  The
 //    eigenpairs of a 3x3 C take FP64 for a fifth of their operations (eig3_split): 160^3 seeds 6.23 ->
-//    2.12 ms at three blocks per SM (2.25 ms at two), the FP64 pipe 60% busy;
+//    2.12 ms at three blocks per SM (2.25 ms at two), the FP64 pipe 82% busy;
 //  * the FTLE, an FP32 output: the same formulas in double-FP32 (dfloat_device.cuh), about 200 FP32
 //    operations per seed in 2D and 700 in 3D in place of 65 and 170 FP64 ones, whether or not C or
 //    lambda_max is asked for (one call's FTLE does not depend on its other outputs).  Auxiliary
