@@ -92,8 +92,11 @@ __global__ void __launch_bounds__(256, 3) rk4_tet_kernel(TetDev T, Rk4Args A, co
 // Issue bounds it (23 of 32 lanes active: in most warps some lane leaves its cell at every stage): four blocks
 // of 256 threads (27.8 ms on the 1.6M-triangle stenosis, 4096 x 1024 seeds, 500 steps; five: 31.8, three:
 // 31.0), both components in two-lane FP32 instructions (28.3 without).
-template <int ST>
-__global__ void __launch_bounds__(256, 4) rk4_tri_kernel(TriDev T, Rk4Args A, const int *__restrict__ cells0,
+// PACK false: few tracers, whose steps are one dependent chain: without the two-lane instructions and with
+// registers for two blocks per SM (84, no spills): 16,384 seeds 2.94 against 3.05 ms, 65,536 2.51 / 2.60, 131,072
+// 2.78 / 2.33.
+template <int ST, bool PACK>
+__global__ void __launch_bounds__(256, PACK ? 4 : 2) rk4_tri_kernel(TriDev T, Rk4Args A, const int *__restrict__ cells0,
                                                       unsigned *errword)
 {
     const long long i = thread_tracer(A);
@@ -125,12 +128,12 @@ __global__ void __launch_bounds__(256, 4) rk4_tri_kernel(TriDev T, Rk4Args A, co
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             const float c = s == 0 ? 0.0f : (s == 3 ? h : hh);
-            const float2 z = s == 0 ? x : __ffma2_rn(make_float2(c, c), k[s == 0 ? 0 : s - 1], x);
+            const float2 z = s == 0 ? x : fma2<PACK>(c, k[s == 0 ? 0 : s - 1], x);
             const float y[2] = {z.x, z.y};
             const SchedEntry &es = e[s == 0 ? 0 : (s == 3 ? 2 : 1)];
             r = tri_locate_cached(T, y, &cell, lam, cc);
             if (r != TET_INSIDE) break;
-            k[s] = tri_interp_cached<ST>(T, cell, es.k, lam, T.pairs + (size_t)es.k * T.fstride, es.a, cc);
+            k[s] = tri_interp_cached<ST, PACK>(T, cell, es.k, lam, T.pairs + (size_t)es.k * T.fstride, es.a, cc);
         }
         if (r != TET_INSIDE) {  // a stage point left the mesh: freeze at the start of the step
             st = r == TET_OUTSIDE ? LCS_TRACER_LEFT : LCS_TRACER_WALKFAIL;
@@ -139,7 +142,12 @@ __global__ void __launch_bounds__(256, 4) rk4_tri_kernel(TriDev T, Rk4Args A, co
             break;
         }
         const float h6 = h * (1.0f / 6.0f);
-        rk4_advance2(x, cx, h6, k[0], k[1], k[2], k[3]);
+        if constexpr (PACK) {
+            rk4_advance2(x, cx, h6, k[0], k[1], k[2], k[3]);
+        } else {
+            rk4_advance(x.x, cx.x, h6, k[0].x, k[1].x, k[2].x, k[3].x);
+            rk4_advance(x.y, cx.y, h6, k[0].y, k[1].y, k[2].y, k[3].y);
+        }
         for (; si < A.nsnap && snap_step(A, si, ns) == n + 1; ++si)
             store(snap_slot(A, job, si), snap_exit(A, job, si, st, te));
     }
@@ -601,12 +609,16 @@ cudaError_t launch_rk4_tet(lcs_ctx *ctx, const Rk4Launch &L, const int *cells0, 
     if (f->kind == LCS_TRI) {
         const TriDev T = tri_dev(f, walk_limit);
         lcs_tm_begin(ctx, 0, s);
-        if (f->storage == LCS_F32)
-            rk4_tri_kernel<LCS_F32><<<grid, bt, 0, s>>>(T, A, cells0, ctx->d_errword);
-        else if (f->storage == LCS_F16)
-            rk4_tri_kernel<LCS_F16><<<grid, bt, 0, s>>>(T, A, cells0, ctx->d_errword);
-        else
-            rk4_tri_kernel<LCS_BF16><<<grid, bt, 0, s>>>(T, A, cells0, ctx->d_errword);
+        const bool few = L.N * L.njobs <= 512LL * ctx->num_sms;   // all resident in two blocks per SM
+#define TRI_LAUNCH(ST)                                                                             \
+    do {                                                                                           \
+        if (few) rk4_tri_kernel<ST, false><<<grid, bt, 0, s>>>(T, A, cells0, ctx->d_errword);      \
+        else rk4_tri_kernel<ST, true><<<grid, bt, 0, s>>>(T, A, cells0, ctx->d_errword);           \
+    } while (0)
+        if (f->storage == LCS_F32) TRI_LAUNCH(LCS_F32);
+        else if (f->storage == LCS_F16) TRI_LAUNCH(LCS_F16);
+        else TRI_LAUNCH(LCS_BF16);
+#undef TRI_LAUNCH
         lcs_tm_end(ctx, 0, s);
         return cudaGetLastError();
     }

@@ -217,14 +217,28 @@ struct TriPair<LCS_BF16> {
 // u = sum_i lam_i [(1 - a) u_k + a u_{k+1}](vertex i) from the vertices' pairs (u_k, u_{k+1}).
 // Every pair holds finite values (a single frame is paired with itself), so a = 0 gives u_k
 // exactly without a select: 0 * u_{k+1} + 1 * u_k.
-// Both components go through the two-lane FP32 instructions.
+// PACK: both components through the two-lane FP32 instructions, else one after the other (the same bits).
+template <bool PACK>
+__device__ __forceinline__ float2 fma2(float a, float2 b, float2 c)
+{
+    if constexpr (PACK) return __ffma2_rn(make_float2(a, a), b, c);
+    else return make_float2(__fmaf_rn(a, b.x, c.x), __fmaf_rn(a, b.y, c.y));
+}
+
+template <bool PACK>
+__device__ __forceinline__ float2 mul2(float a, float2 b)
+{
+    if constexpr (PACK) return __fmul2_rn(make_float2(a, a), b);
+    else return make_float2(__fmul_rn(a, b.x), __fmul_rn(a, b.y));
+}
+
+template <bool PACK = true>
 __device__ __forceinline__ float2 tri_blend(const float *lam, const float2 *ua, const float2 *ub, float a)
 {
-    const float2 a2 = make_float2(a, a), g2 = make_float2(1.0f - a, 1.0f - a);
+    const float g = 1.0f - a;
     float2 acc = make_float2(0.0f, 0.0f);
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-        acc = __ffma2_rn(make_float2(lam[i], lam[i]), __ffma2_rn(a2, ub[i], __fmul2_rn(g2, ua[i])), acc);
+    for (int i = 0; i < 3; ++i) acc = fma2<PACK>(lam[i], fma2<PACK>(a, ub[i], mul2<PACK>(g, ua[i])), acc);
     return acc;
 }
 
@@ -243,7 +257,7 @@ __device__ __forceinline__ void tri_interp(const TriDev &T, int c, const float *
 }
 
 // tri_interp in interval k (pairs at fp) with the vertex pairs taken from, or put into, the cache
-template <int ST>
+template <int ST, bool PACK = true>
 __device__ __forceinline__ float2 tri_interp_cached(const TriDev &T, int c, int k, const float *lam, const char *fp,
                                                     float a, TriCache &cc)
 {
@@ -255,7 +269,7 @@ __device__ __forceinline__ float2 tri_interp_cached(const TriDev &T, int c, int 
         cc.pc = c;
         cc.pk = k;
     }
-    return tri_blend(lam, cc.ua, cc.ub, a);
+    return tri_blend<PACK>(lam, cc.ua, cc.ub, a);
 }
 
 // tri_interp's u plus the Jacobian of the P1 interpolant, constant in the triangle, with c's map m
