@@ -459,9 +459,9 @@ __device__ __forceinline__ int axis_cell_ext(const RectParams &P, const SliceGeo
 }
 
 // Extended cell e and fraction f of x on every axis, as axis_cell_ext gives them.  PM >= 0 (boxes whose axes
-// all wrap, or all end, of at most FLOOR_MAX_NODES nodes): the floor without the conversion pipe, x and y in
-// two-lane FP32 instructions; an index that is out of range, which includes every coordinate beyond the reach
-// of that floor, goes back to axis_cell_ext's floor and wraps.
+// all wrap, or all end, within the reach of floor_index: box3_mask): the floor without the conversion pipe, x and y
+// in two-lane FP32 instructions; an index that is out of range, which includes every coordinate beyond that
+// reach, goes back to axis_cell_ext's floor and wraps.
 template <int PM>
 __device__ __forceinline__ void cell_ext(const RectParams &P, const SliceGeom &G, const float *x, int *e, float *f)
 {
@@ -988,8 +988,7 @@ static cudaError_t episodes(const RectParams &P, const lcs_field *f, const Rk4Ar
             lcs_tm_begin(L.ctx, 0, s);
             // compile-time periodicity for the common all-periodic and non-periodic boxes
             // (of axes within the reach of the kernels' floor)
-            const bool reach = P.n[0] <= FLOOR_MAX_NODES && P.n[1] <= FLOOR_MAX_NODES && P.n[2] <= FLOOR_MAX_NODES;
-            const int pm = reach ? P.periodic[0] | (P.periodic[1] << 1) | (P.periodic[2] << 2) : -1;
+            const int pm = box3_mask(P);
             unsigned *kk = last ? nullptr : keys;
 #define EP_VAR(PM, LAY) \
     ep_var3_kernel<PM, LAY><<<agrid, abt, 0, s>>>(P, G, slices, ss, smap, A, SB, MB, job, s0, s1, shift, kk, hist)

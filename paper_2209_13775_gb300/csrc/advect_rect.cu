@@ -160,9 +160,9 @@ __global__ void __launch_bounds__(256) rk4_gather2_kernel(RectParams P, const ch
 // ------------------------------------------------------------ 3D gather
 
 // Cell i0 (each axis' lower node) and fraction f of x, as axis_cell gives them.  PM >= 0 (boxes whose axes all
-// wrap, or all end, of at most FLOOR_MAX_NODES nodes): the floor without the conversion pipe, x and y in
-// two-lane FP32 instructions; indices more than a period away, which include every coordinate beyond the
-// reach of that floor, go back to floorf.
+// wrap, or all end, within the reach of floor_index: box3_mask): the floor without the conversion pipe, x and y in
+// two-lane FP32 instructions; indices more than a period away, which include every coordinate beyond that
+// reach, go back to floorf.
 template <int PM>
 __device__ __forceinline__ void cell3(const RectParams &P, const float *x, int *i0, float *f)
 {
@@ -213,14 +213,6 @@ __device__ __forceinline__ void cell3(const RectParams &P, const float *x, int *
             axis_cell<PM>(P, d, x[d], i0[d], i1, f[d]);
         }
     }
-}
-
-// periodicity mask of a 3D box whose axes lie within the reach of cell3's floor, or -1
-static int box3_mask(const RectParams &P)
-{
-    for (int d = 0; d < 3; ++d)
-        if (P.n[d] > FLOOR_MAX_NODES) return -1;
-    return (P.periodic[0] ? 1 : 0) | (P.periodic[1] ? 2 : 0) | (P.periodic[2] ? 4 : 0);
 }
 
 // The corners of a tracer's last cell, blended to the time of its last stage (k, a)

@@ -200,10 +200,21 @@ __device__ __forceinline__ void axis_cell(const RectParams &P, int d, float x, i
 // Floor of s as a float and an index without the conversion pipe (float-to-int and int-to-float issue
 // at an eighth of the FP32 rate): t = s + 3 * 2^22 rounded down carries floor(s) in its low mantissa
 // bits for |s| < 2^22.  floor_index of such a t is floor(s); for any larger |s|, infinities and NaN it
-// lies outside [-2^22, 2^22), so a bounds check of the index (axes of at most 2^22 nodes) finds them.
+// lies outside [-2^22, 2^22), but it is not floor(s) there (from t = 2^24 on it counts every second cell).
+// So a closed axis, whose query is clamped to its nodes first, may have FLOOR_MAX_NODES of them; a periodic
+// one only half as many: an index in the next period is taken as it is (less n), and must be below 2^22.
 #define FLOOR_MAGIC 12582912.0f
 #define FLOOR_MAX_NODES (1 << 22)
+#define FLOOR_MAX_PERIODIC (1 << 21)
 __device__ __forceinline__ int floor_index(float t) { return __float_as_int(t) - 0x4b400000; }
+
+// periodicity mask of a 3D box whose axes lie within the reach of that floor, or -1
+static inline int box3_mask(const RectParams &P)
+{
+    for (int d = 0; d < 3; ++d)
+        if (P.n[d] > (P.periodic[d] ? FLOOR_MAX_PERIODIC : FLOOR_MAX_NODES)) return -1;
+    return (P.periodic[0] ? 1 : 0) | (P.periodic[1] ? 2 : 0) | (P.periodic[2] ? 4 : 0);
+}
 
 // 2D box: the constants of axis_cell for both axes, packed for the two-lane FP32 instructions
 struct Box2 {
