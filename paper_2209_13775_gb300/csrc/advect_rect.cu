@@ -1083,6 +1083,7 @@ static cudaError_t launch_slice2d(const RectParams &P, const lcs_field *f, const
         const long long runs = (3LL * A.nsteps_max + FILL_RUN - 1) / FILL_RUN;
         const dim3 fgrid((unsigned)((nodes + 255) / 256), (unsigned)(runs < 65535 ? runs : 65535), (unsigned)L.njobs);
         const char *fr = (const char *)f->d_frames;
+        lcs_tm_begin(L.ctx, 2, s);
 #define FILL(ST)                                                                                                      \
     slice2d_fill_kernel<ST><<<fgrid, 256, 0, s>>>(P, fr, f->frame_stride, A.sched, A.nsteps_max, A.job_nsteps, O,    \
                                                   (int)nodes, shared, slices)
@@ -1090,8 +1091,8 @@ static cudaError_t launch_slice2d(const RectParams &P, const lcs_field *f, const
         else if (f->storage == LCS_F16) FILL(LCS_F16);
         else FILL(LCS_BF16);
 #undef FILL
+        lcs_tm_end(L.ctx, 2, s);
     }
-    lcs_tm_end(L.ctx, 2, s);
     lcs_tm_begin(L.ctx, 0, s);
     dim3 grid(seed_map_grid(A.map, A.N, bt), (unsigned)L.njobs);
     const int pm = P.periodic[0] | (P.periodic[1] << 1);
