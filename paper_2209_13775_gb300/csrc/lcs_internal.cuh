@@ -273,12 +273,25 @@ struct Rk4Launch {
 //     400 steps: 64^3: 512,000 6.3 / 6.9, 778,688 9.6 / 8.5; 128^3: 2.1M 28.3 / 29.8, 2.7M 37.4 / 35.7
 //   variational (bound by issue), FP32, 100 steps: 64^3: 512,000 2.03 / 2.33, 1M 3.98 / 3.84; 128^3: 2.1M
 //     8.4 / 9.5, 4.1M 16.0 / 16.3; 400 steps: 64^3: 262,144 5.4 / 5.8, 512,000 9.6 / 9.1; 128^3: 1M 21.9 / 22.2
+// Boxes periodic along some axes only, whose cell search is the general one in both (periodic along x and z; ABC
+// flow, one-pass / re-bundled):
+//   FP32, 100 steps: 64^3 nodes: 512,000 seeds 1.47 / 1.50, 778,688 2.24 / 1.90; 128^3: 1.8M 5.25 / 5.74, 2.6M 7.34 /
+//     7.14; 400 steps: 64^3: 262,144 3.08 / 3.41, 373,248 3.99 / 3.87; 128^3: 1.3M 13.5 / 14.1, 1.8M 17.8 / 16.1
+//   FP16, 100 steps: 64^3: 512,000 1.37 / 1.50, 778,688 2.12 / 1.89; 128^3: 2.6M 6.85 / 7.08, 4.1M 9.87 / 9.56;
+//     400 steps: 64^3: 373,248 3.50 / 3.89, 512,000 4.47 / 4.38; 128^3: 1.8M 15.2 / 15.9, 2.6M 20.9 / 19.3
+//   variational: 100 steps: 64^3: 778,688 3.42 / 3.72; 128^3: 4.1M 16.4 / 18.6: as on other boxes
 static inline long long rk4_rebundle_seeds(const lcs_field *f, bool variational, int steps)
 {
     const long long nodes = (long long)f->n[0] * f->n[1] * f->n[2];
     const bool half = f->storage != LCS_F32 && !variational;
-    const long long at100 = (1LL << 19) + (half || variational ? 2 * nodes : nodes);
-    const int longest = half ? 200 : 300, s = steps < 100 ? 100 : steps > longest ? longest : steps;
+    const int axes = f->periodic[0] + f->periodic[1] + f->periodic[2];
+    long long at100 = (1LL << 19) + (half || variational ? 2 * nodes : nodes);
+    int longest = half ? 200 : 300;
+    if ((axes == 1 || axes == 2) && !variational) {
+        at100 = (1LL << 18) + (half ? nodes * 7 / 5 : nodes);
+        longest = half ? 130 : 200;
+    }
+    const int s = steps < 100 ? 100 : steps > longest ? longest : steps;
     const long long n = at100 * 100 / s;
     return n > (1LL << 18) ? n : 1LL << 18;
 }
