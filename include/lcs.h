@@ -459,7 +459,8 @@ lcs_status lcs_cauchy_green(lcs_ctx *ctx, const lcs_flowmap *fm, int job, double
 
 /* FTLE sigma = ln(sqrt(lambda_max(C))) / |T| (Sec. 1: the FTLE is derived from
  * the largest eigenvalue of C) as FP32 [N], NaN where C is undefined, computed
- * with 46-bit arithmetic from the FP32 positions whatever else is asked for;
+ * from the FP32 positions, whatever else is asked for, in double-FP32 arithmetic
+ * where the eigenvalue's error stays below 2^-30 of its logarithm and in FP64 elsewhere;
  * optionally lambda_max [N] FP64 and C (as lcs_cauchy_green) from the same
  * pass.  lambda_max and C may be NULL.  job = -1 writes every job.
  * Errors: as lcs_cauchy_green.                                              */

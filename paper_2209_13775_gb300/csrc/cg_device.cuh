@@ -548,9 +548,9 @@ static __device__ __noinline__ float ftle_from_c64(const double *C, float half_i
 }
 
 // sigma = ln(lambda_max(G^T G)) * half_inv_T with G in double-FP32 (its entries' magnitudes between
-// 2^-40 and 2^40 at the largest: nothing below then leaves the FP32 range)
+// 2^-40 and 2^40 at the largest: nothing below then leaves the FP32 range); false where sigma needs FP64
 template <int DIM>
-__device__ __forceinline__ float ftle_from_grad32(const dfl (*G)[DIM], float half_inv_T)
+__device__ __forceinline__ bool ftle_from_grad32(const dfl (*G)[DIM], float half_inv_T, float *sigma)
 {
     constexpr int NP = DIM == 2 ? 3 : 6;
     dfl C[NP];
@@ -564,17 +564,13 @@ __device__ __forceinline__ float ftle_from_grad32(const dfl (*G)[DIM], float hal
             for (int a = 1; a < DIM; ++a) s = df_add(s, df_mul(G[a][i], G[a][j]));
             C[o++] = s;
         }
-    if constexpr (DIM == 2) {
-        return df_log(df_eig_max2(C)) * half_inv_T;
-    } else {
-        bool ok;
-        const dfl lm = df_eig_max3(C, &ok);
-        if (ok) return df_log(lm) * half_inv_T;
-        double Cd[6];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) Cd[q] = df_to_double(C[q]);
-        return ftle_from_c64<3>(Cd, half_inv_T);
-    }
+    float gap = 1.0f, ln;
+    if constexpr (DIM == 2)
+        ln = df_log(df_eig_max2(C));
+    else
+        ln = df_log(df_eig_max3(C, &gap));
+    *sigma = ln * half_inv_T;
+    return fabsf(ln) * gap >= 0x1p-14f;   // 2^-44 / gap of lambda_max is at most 2^-30 of its logarithm
 }
 
 // whether G's largest entry lies where ftle_from_grad32 is safe (false for NaN and infinite entries)
@@ -594,7 +590,7 @@ __device__ __forceinline__ bool grad32_in_range(const dfl (*G)[DIM])
 }
 
 // FTLE of a seed from its positions f[b][k][a] (axis b, point k = 0 the seed, 1 and 2 the two others,
-// component a) in double-FP32, in FP64 where grad F lies outside the safe range
+// component a) in double-FP32, in FP64 where grad F lies outside the safe range or sigma needs it
 template <int DIM>
 __device__ __forceinline__ float ftle_from_positions(const CgLaunch &L, const AxisDiff *d, const float *f0,
                                                      const float (*f1)[DIM], const float (*f2)[DIM], float half_inv_T)
@@ -608,7 +604,8 @@ __device__ __forceinline__ float ftle_from_positions(const CgLaunch &L, const Ax
 #pragma unroll
     for (int b = 0; b < DIM; ++b) none |= d[b].mode == 0;
     if (none) return __int_as_float(0x7fc00000);
-    if (L.df_ok && grad32_in_range<DIM>(G)) return ftle_from_grad32<DIM>(G, half_inv_T);
+    float sigma;
+    if (L.df_ok && grad32_in_range<DIM>(G) && ftle_from_grad32<DIM>(G, half_inv_T, &sigma)) return sigma;
     double G64[DIM][DIM], C[DIM == 2 ? 3 : 6];
 #pragma unroll
     for (int b = 0; b < DIM; ++b)

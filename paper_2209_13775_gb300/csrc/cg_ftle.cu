@@ -126,9 +126,7 @@ __global__ void __launch_bounds__(256, EIG ? 3 : 1) cg_ftle_kernel(const __grid_
 #pragma unroll
                 for (int b = 0; b < DIM; ++b) Gf[a][b] = {M[a][b], 0.0f};
             float s = __int_as_float(0x7fc00000);
-            if (grad32_in_range<DIM>(Gf)) {
-                s = ftle_from_grad32<DIM>(Gf, half_inv_T);
-            } else if (ok) {
+            if (ok && !(grad32_in_range<DIM>(Gf) && ftle_from_grad32<DIM>(Gf, half_inv_T, &s))) {
                 double C[NP];
 #pragma unroll
                 for (int a = 0; a < DIM; ++a)

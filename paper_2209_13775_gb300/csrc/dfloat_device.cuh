@@ -3,9 +3,11 @@
 //
 // GB300 issues 128 FP32 operations per SM and cycle and 2 FP64 ones, so a chain of FP32 operations
 // that stands in for an FP64 one is worth taking wherever the result does not have to carry 53 bits.
-// The FTLE is such a result: it is an FP32 value, the logarithm of an eigenvalue whose relative
-// error here stays near 2^-45, 2^21 times below the rounding of the stored value.  lcs_ftle's
-// lambda_max and C, which are FP64 outputs, do not come from here.
+// The FTLE is such a result: it is an FP32 value, the logarithm of an eigenvalue whose relative error
+// here, from the positions on, is at most 2^-44 (2^-44.5 over 6M gradients in random orientations), and
+// 2^-44 / sqrt(d) where the two largest eigenvalues come together (d: df_eig_max3).  The caller takes FP64
+// wherever that exceeds 2^-30 of the logarithm, a thirty-second of the half ulp by which the stored value is
+// rounded.  lcs_ftle's lambda_max and C, which are FP64 outputs, do not come from here.
 //
 // The sums and products are the error-free transformations of Knuth (TwoSum), Dekker (Fast2Sum)
 // and the FMA residual of a product, written with round-to-nearest intrinsics so that no product
@@ -75,18 +77,6 @@ __device__ __forceinline__ dfl df_sqrt(dfl a)
     return df_fast_sum(s, __fdividef(__fadd_rn(__fmaf_rn(-s, s, a.h), a.l), s + s));
 }
 
-// sum of n products
-template <int N>
-__device__ __forceinline__ dfl df_dot(const dfl *a, const dfl *b)
-{
-    dfl s = df_mul(a[0], b[0]);
-#pragma unroll
-    for (int i = 1; i < N; ++i) s = df_add(s, df_mul(a[i], b[i]));
-    return s;
-}
-
-__device__ __forceinline__ double df_to_double(dfl a) { return (double)a.h + (double)a.l; }
-
 // the power of two 2^-e (and its inverse) that takes x = m 2^e into [1, 2); x normal
 __device__ __forceinline__ float df_inv_pow2(float x, float &pow2)
 {
@@ -110,9 +100,9 @@ __device__ __forceinline__ dfl df_eig_max2(const dfl *C)
 // d = 1 - |r| and t the root in [0, 2 - sqrt 3] of 9 t - 6 t^2 + t^3 = 2 d (simple everywhere, its
 // slope 3 (1 - t)(3 - t) is at least 5.9), beta = 2 - t for r >= 0; for r < 0 the isolated root is
 // t - 2 and beta the larger root of the quadratic that is left, 1 - t/2 + sqrt(3 t (4 - t)) / 2.
-// An error e of r moves that root by about e / sqrt(6 d): at d >= 1e-9 below 1e-9.  Below (the two
-// largest eigenvalues within 3e-5 p of each other) *ok is cleared: the caller takes Jacobi rotations.
-__device__ __forceinline__ dfl df_eig_max3(const dfl *C, bool *ok)
+// An error e of r moves that root by about e / sqrt(6 d): *gap is sqrt(d), 1 for r >= 0, and 0 below
+// d = 1e-9, where d itself has lost its digits.  (0.25: all three eigenvalues within 2e-13 of q.)
+__device__ __forceinline__ dfl df_eig_max3(const dfl *C, float *gap)
 {
     float is;
     const float s = df_inv_pow2(fmaxf(C[0].h, fmaxf(C[3].h, C[5].h)), is);
@@ -124,7 +114,7 @@ __device__ __forceinline__ dfl df_eig_max3(const dfl *C, bool *ok)
     const dfl off = df_add(df_add(df_mul(a01, a01), df_mul(a02, a02)), df_mul(a12, a12));
     const dfl dia = df_add(df_add(df_mul(b00, b00), df_mul(b11, b11)), df_mul(b22, b22));
     const dfl p2 = df_mul(df_add(dia, df_scale(off, 2.0f)), df_scale(third, 0.5f));
-    *ok = true;
+    *gap = p2.h >= 1e-26f ? 1.0f : 0.25f;
     if (!(p2.h >= 1e-26f)) return df_scale(q, is);   // all eigenvalues within 2e-13 of q (NaN: q is NaN)
     // y = 1 / sqrt(p2): FP32 estimate and one step from its exact residual
     const float y0 = rsqrtf(p2.h);
@@ -143,7 +133,7 @@ __device__ __forceinline__ dfl df_eig_max3(const dfl *C, bool *ok)
     const bool neg = r.h < 0.0f;
     dfl d = df_add(neg ? r : df_neg(r), 1.0f);
     if (d.h < 0.0f) d = {0.0f, 0.0f};   // |r| above 1 by rounding
-    if (neg && d.h < 1e-9f) *ok = false;
+    if (neg) *gap = d.h < 1e-9f ? 0.0f : sqrtf(d.h);
     // t in FP32 (two Newton steps from the start of its series), then one step in double-FP32
     const float c = d.h * (2.0f / 9.0f);
     float t0 = c * fmaf(2.0f / 3.0f, c, 1.0f);
