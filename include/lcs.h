@@ -391,6 +391,15 @@ lcs_status lcs_mlp_set_params(lcs_ctx *ctx, lcs_mlp *mlp, const float *params, i
 lcs_status lcs_mlp_get_params(lcs_ctx *ctx, const lcs_mlp *mlp, float *params, int on_device);
 void lcs_mlp_free(lcs_mlp *mlp);
 
+/* Seconds a block of the network's kernels (lcs_mlp_forward, lcs_mlp_loss_grad,
+ * training, surrogate steps) waits for the copy of the weights before it gives up
+ * and the next lcs_synchronize reports LCS_ETIMEOUT (the results of that call are
+ * then incomplete); 0 = 1 s (the default), at most 60 s; under 1e-6 a copy not
+ * complete at its first test counts as late.  A copy already issued is always
+ * waited for (with the 1 s bound) before a block exits.
+ * Errors: LCS_EINVAL.                                                        */
+lcs_status lcs_mlp_set_wait_limit(lcs_ctx *ctx, lcs_mlp *mlp, double seconds);
+
 /* Outputs o [3][n] (o0, o1, o2 rows) at points xyt [3][n] (x, y, t rows).    */
 lcs_status lcs_mlp_forward(lcs_ctx *ctx, const lcs_mlp *mlp, long long n, const float *xyt, float *out,
                            int on_device);

@@ -125,6 +125,15 @@ extern "C" void lcs_mlp_free(lcs_mlp *m)
     delete m;
 }
 
+extern "C" lcs_status lcs_mlp_set_wait_limit(lcs_ctx *ctx, lcs_mlp *m, double seconds)
+{
+    if (!ctx) return LCS_EINVAL;
+    if (!m || !(seconds >= 0.0 && seconds <= 60.0))
+        return lcs_fail(ctx, LCS_EINVAL, "lcs_mlp_set_wait_limit: null network or a limit outside 0..60 s");
+    m->wait_ns = seconds > 0.0 ? (unsigned long long)(seconds * 1e9) : LCS_WAIT_LIMIT_NS;
+    return LCS_OK;
+}
+
 extern "C" lcs_status lcs_mlp_forward(lcs_ctx *ctx, const lcs_mlp *m, long long n, const float *xyt, float *out,
                                       int on_device)
 {
@@ -161,6 +170,7 @@ extern "C" lcs_status lcs_mlp_forward(lcs_ctx *ctx, const lcs_mlp *m, long long 
     A.out1 = dst + n;
     A.out2 = dst + 2 * n;
     A.errword = ctx->d_errword;
+    A.wait_ns = m->wait_ns;
     cudaError_t e = launch_mlp_step(A, ctx->num_sms, ctx->stream);
     if (e == cudaSuccess && !on_device)
         e = cudaMemcpyAsync(out, dout, sizeof(float) * 3 * n, cudaMemcpyDeviceToHost, ctx->stream);
@@ -261,6 +271,7 @@ lcs_status advect_surrogate(lcs_ctx *ctx, const lcs_field *f, const lcs_seeds *s
         A.out1 = xp + N;
         A.out2 = xp + 2 * N;
         A.errword = ctx->d_errword;
+        A.wait_ns = m->wait_ns;
         lcs_tm_begin(ctx, 0, ctx->stream);
         e = launch_mlp_step(A, ctx->num_sms, ctx->stream);
         lcs_tm_end(ctx, 0, ctx->stream);

@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __nv_bfloat16 *__r
         __syncthreads();
         if (abort_flag) break;
     }
+    if (abort_flag) mbar_wait_bounded(&bar, phase ^ 1);   // the wait gave up: the MMAs in flight end first
     tc_fence_after();
     if (!abort_flag && !first) {
         const long long row = m0 + warp * 32 + lane;

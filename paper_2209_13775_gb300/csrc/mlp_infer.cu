@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(NG * 128, 1) mlp_step_kernel(const MlpStepArgs
         mbar_arrive_expect_tx(&bar_w, MLP_TILE_BYTES);
         bulk_g2s(smem, A.tiles, MLP_TILE_BYTES, &bar_w);
     }
-    const bool have_w = !__syncthreads_or(!tc_wait(&bar_w, 0, A.errword));
+    const bool have_w = !__syncthreads_or(!tc_wait(&bar_w, 0, A.errword, A.wait_ns));
     const uint32_t tmem = tmem_base + TM_ACC + (uint32_t)(g * NS);
     unsigned char *sAct = smem + OFF_WG + g * WG_BYTES;
     unsigned char *sPhi = sAct + ACT_BYTES;
@@ -232,6 +232,8 @@ __global__ void __launch_bounds__(NG * 128, 1) mlp_step_kernel(const MlpStepArgs
         }
         wg_sync(g);   // the outputs are read before the next tile's features take their place
     }
+    if (!have_w) mbar_wait_bounded(&bar_w, 0);         // a wait gave up: what is in flight ends first
+    else if (abort_flag[g]) mbar_wait_bounded(&bar_g[g], phase ^ 1);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_free(tmem_base, 512);

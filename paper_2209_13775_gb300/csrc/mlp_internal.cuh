@@ -40,6 +40,7 @@ struct lcs_mlp {
     float *d_grad = nullptr;          // gradient [MLP_NPARAMS]
     void *d_work = nullptr;           // trainer's partial gradients
     double *d_loss = nullptr;         // summed loss of the last lcs_mlp_loss_grad
+    unsigned long long wait_ns = LCS_WAIT_LIMIT_NS;  // bound on a block's wait for the weights (lcs_mlp_set_wait_limit)
 };
 
 #ifdef __CUDACC__
@@ -78,6 +79,7 @@ struct MlpStepArgs {
     int mode;                 // 0: out = (o0, o1, o2); 1: out = (x + s o0, y + s o1, o2)
     float *out0, *out1, *out2;
     unsigned *errword;
+    unsigned long long wait_ns;  // bound on a block's wait for the weights
 };
 
 struct SurGateArgs {

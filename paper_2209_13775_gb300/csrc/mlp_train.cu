@@ -69,6 +69,7 @@ struct TrainArgs {
     float *part;                       // [CTAs][PART_STRIDE] partial gradients
     double *part_loss;                 // [CTAs]
     unsigned *errword;
+    unsigned long long wait_ns;        // bound on a CTA's wait for the weights
 };
 
 constexpr int TN = 96;                 // samples per tile
@@ -133,7 +134,8 @@ __global__ void __launch_bounds__(256, 1) train_step_kernel(const TrainArgs A)
     for (int q = tid; q < 16 * TN / 8; q += 256) {    // rows 3..15 of dO stay zero
         *reinterpret_cast<uint4 *>(smem + DO_OFF + 16 * q) = make_uint4(0, 0, 0, 0);
     }
-    bool ok = !__syncthreads_or(!tc_wait(&bar_w, 0, A.errword));
+    const bool have_w = !__syncthreads_or(!tc_wait(&bar_w, 0, A.errword, A.wait_ns));
+    bool ok = have_w;
     const uint32_t tm = tmem_base, us = smem_u32(smem);
     const uint32_t tw = tm + TM_WORK + ((uint32_t)((warp & 3) * 32) << 16) + TH * g;   // this thread's lane and columns
     const float *bias = reinterpret_cast<const float *>(smem + BIAS_OFF);
@@ -374,6 +376,11 @@ __global__ void __launch_bounds__(256, 1) train_step_kernel(const TrainArgs A)
 #pragma unroll
             for (int j = 0; j < 3; ++j) out[P_DB4 + j] = (red_g[0][j] + red_g[1][j]) + (red_g[2][j] + red_g[3][j]);
         }
+    } else if (!have_w) {                             // a wait gave up: what is in flight ends first
+        mbar_wait_bounded(&bar_w, 0);
+    } else {
+        if (tid == 0) tc_commit(&bar);                // behind MMAs issued since the commit that was waited for
+        if (mbar_wait_bounded(&bar, phase ^ 1)) mbar_wait_bounded(&bar, phase);
     }
     tc_fence_before();
     __syncthreads();
@@ -528,6 +535,7 @@ cudaError_t mlp_loss_grad(lcs_mlp *m, const float *xyt, long long xstride, const
     A.part_loss = (double *)m->d_work;
     A.part = (float *)(A.part_loss + num_sms);
     A.errword = errword;
+    A.wait_ns = m->wait_ns;
     const long long tiles = (B + TN - 1) / TN;
     const int grid = (int)(tiles < num_sms ? tiles : num_sms);
     train_step_kernel<<<grid, 256, TRAIN_SMEM, s>>>(A);

@@ -111,10 +111,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v)
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// wait for an mbarrier phase with the library's time bound; on timeout set the error bit
-__device__ __forceinline__ bool tc_wait(uint64_t *bar, unsigned parity, unsigned *errword)
+// wait for an mbarrier phase with a time bound (the library's, if none is given); on timeout set the error bit.  A
+// block that gives up then waits once more, with the library's bound, for whatever it has in flight before it leaves
+// its shared and tensor memory to the next block.
+__device__ __forceinline__ bool tc_wait(uint64_t *bar, unsigned parity, unsigned *errword,
+                                        uint64_t limit_ns = LCS_WAIT_LIMIT_NS)
 {
-    if (mbar_wait_bounded(bar, parity)) return true;
+    if (mbar_wait_limit(bar, parity, limit_ns)) return true;
     atomicOr(errword, LCS_ERRBIT_TIMEOUT);
     return false;
 }

@@ -33,6 +33,7 @@ EXPORTS = ["lcs_create", "lcs_destroy", "lcs_last_error", "lcs_set_stream", "lcs
            "lcs_timing_read",
            "lcs_advect_rk4_noalloc", "lcs_gemm_bf16", "lcs_mlp_create", "lcs_mlp_set_params",
            "lcs_mlp_get_params", "lcs_mlp_free", "lcs_mlp_forward", "lcs_mlp_loss_grad", "lcs_mlp_adam",
+           "lcs_mlp_set_wait_limit",
            "lcs_surrogate_train", "lcs_context_device", "lcs_field_dim"]
 PHASE_ADVECT, PHASE_REBUNDLE, PHASE_SLICES, PHASE_CG = 0, 1, 2, 3
 NOALLOC_MAX_STEPS = 43680
@@ -109,7 +110,7 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
         "lcs_gemm_bf16": ([P, LL, I, LL, P, LL, P, LL, P, LL, I, I], S),
         "lcs_mlp_create": ([P, P, P, I, P], S), "lcs_mlp_set_params": ([P, P, P, I], S),
         "lcs_mlp_get_params": ([P, P, P, I], S), "lcs_mlp_free": ([P], None),
-        "lcs_mlp_forward": ([P, P, LL, P, P, I], S),
+        "lcs_mlp_set_wait_limit": ([P, P, ctypes.c_double], S), "lcs_mlp_forward": ([P, P, LL, P, P, I], S),
         "lcs_mlp_loss_grad": ([P, P, LL, P, P, ctypes.c_double, P, P, I], S),
         "lcs_mlp_adam": ([P, P, P, I, ctypes.c_double, ctypes.c_double, ctypes.c_double, ctypes.c_double], S),
         "lcs_surrogate_train": ([P, P, P, P, LL, P, I, P], S),
@@ -507,6 +508,10 @@ def lcs_mlp_get_params(ctx, mlp, params):
 
 def lcs_mlp_free(mlp):
     load().lcs_mlp_free(mlp)
+
+
+def lcs_mlp_set_wait_limit(ctx, mlp, seconds):
+    _check(ctx, load().lcs_mlp_set_wait_limit(ctx, mlp, float(seconds)))
 
 
 def lcs_mlp_forward(ctx, mlp, xyt, out):
