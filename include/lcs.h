@@ -394,7 +394,8 @@ void lcs_mlp_free(lcs_mlp *mlp);
 /* Seconds a block of the network's kernels (lcs_mlp_forward, lcs_mlp_loss_grad,
  * training, surrogate steps) waits for the copy of the weights before it gives up
  * and the next lcs_synchronize reports LCS_ETIMEOUT (the results of that call are
- * then incomplete); 0 = 1 s (the default), at most 60 s; under 1e-6 a copy not
+ * then incomplete: outputs not written, gradients without the block's samples, the
+ * loss NaN); 0 = 1 s (the default), at most 60 s; under 1e-6 a copy not
  * complete at its first test counts as late.  A copy already issued is always
  * waited for (with the 1 s bound) before a block exits.
  * Errors: LCS_EINVAL.                                                        */

@@ -376,11 +376,17 @@ __global__ void __launch_bounds__(256, 1) train_step_kernel(const TrainArgs A)
 #pragma unroll
             for (int j = 0; j < 3; ++j) out[P_DB4 + j] = (red_g[0][j] + red_g[1][j]) + (red_g[2][j] + red_g[3][j]);
         }
-    } else if (!have_w) {                             // a wait gave up: what is in flight ends first
-        mbar_wait_bounded(&bar_w, 0);
     } else {
-        if (tid == 0) tc_commit(&bar);                // behind MMAs issued since the commit that was waited for
-        if (mbar_wait_bounded(&bar, phase ^ 1)) mbar_wait_bounded(&bar, phase);
+        if (!have_w) {                                // a wait gave up: what is in flight ends first
+            mbar_wait_bounded(&bar_w, 0);
+        } else {
+            if (tid == 0) tc_commit(&bar);            // behind MMAs issued since the commit that was waited for
+            if (mbar_wait_bounded(&bar, phase ^ 1)) mbar_wait_bounded(&bar, phase);
+        }
+        // nothing of an earlier batch is summed in this CTA's place, and the loss tells
+        float4 *out = reinterpret_cast<float4 *>(A.part + (size_t)blockIdx.x * PART_STRIDE);
+        for (int q = tid; q < PART_STRIDE / 4; q += 256) out[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (tid == 0) A.part_loss[blockIdx.x] = __longlong_as_double(0x7ff8000000000000LL);
     }
     tc_fence_before();
     __syncthreads();

@@ -66,8 +66,9 @@ def test_loss_grad(ctx, n):
         loss = lcs.lcs_mlp_loss_grad(ctx, m, xyt, disp, 0.25, g[0])
         lcs.lcs_synchronize(ctx)
         lcs.lcs_mlp_set_wait_limit(ctx, m, 1e-9)
-        lcs.lcs_mlp_loss_grad(ctx, m, xyt, disp, 0.25, g[1])
+        assert np.isnan(lcs.lcs_mlp_loss_grad(ctx, m, xyt, disp, 0.25, g[1]))
         assert timed_out(ctx)
+        assert not g[1].any()         # no block had its weights: nothing, and nothing of the batch before
         lcs.lcs_mlp_set_wait_limit(ctx, m, 0.0)
         assert lcs.lcs_mlp_loss_grad(ctx, m, xyt, disp, 0.25, g[1]) == loss
         lcs.lcs_synchronize(ctx)
