@@ -54,7 +54,7 @@ NSTEPS = int(round(T_END / DT))
 FLOP_PER_TRACER_STEP = 440
 # DRAM read + write bytes per tracer-step of the episode kernel, from the ncu capture of the small case
 # with the same tracer density (profiles/ep_advect3_traffic.md)
-TRAFFIC_BYTES_PER_TRACER_STEP = 23.2
+TRAFFIC_BYTES_PER_TRACER_STEP = 23.7
 
 
 def parse():
@@ -440,9 +440,9 @@ def our_arm(args, rank, world, local):
                      "traffic_note": "ncu DRAM bytes per tracer-step of the small case (64^3 field, 128^3 "
                                      "seeds) scaled by this launch's tracer-steps "
                                      "(profiles/ep_advect3_traffic.md)",
-                     "limiter": "the gathers (ncu, 40-step launch at this size): the L1 data stage 80% busy, its "
-                                "hit rate 55% (the re-bundled tracers spread over 5-8 rows of cells within a few "
-                                "steps), issue 67%, 403 instructions per warp-step, half the warps of an SM "
+                     "limiter": "the gathers (ncu, 40-step launch of the small case): the L1 data stage 76% busy, its "
+                                "hit rate 54% (the re-bundled tracers spread over 5-8 rows of cells within a few "
+                                "steps), issue 66%, 406 instructions per warp-step, half the warps of an SM "
                                 "resident (64 registers)"},
         "phases_ms_per_step": {k: v[0] / args.steps for k, v in phase.items()},
         "clocks": clocks,

@@ -266,8 +266,11 @@ typedef struct {
                                    5 = the field blended once to every stage time of
                                        every job (2D time slices; up to 16 GiB; the
                                        default in 2D when they take at most 2 GiB).
-                                   The default in 3D is 1, and 3 from about as many
-                                   tracers as the field has nodes on (262144 at least) */
+                                   The default in 3D is 1 for few tracers and 3 for
+                                   many, from a count that depends on the nodes, the
+                                   steps of the longest job, the storage type, the
+                                   periodic axes and variational: 262144 at least,
+                                   on 64^3 nodes up to 1 M, on 128^3 up to 4.7 M    */
     const void *surrogate;      /* LCS_SURROGATE: the lcs_mlp to step with            */
     int episode_steps;          /* variant 3: RK4 steps between re-bundlings (0 = 40) */
     int tracers_per_thread;     /* variants 2 and 4: 1 or 2 tracers per thread (0 = 1) */

@@ -277,10 +277,10 @@ __global__ void ep_slice_table_kernel(const SchedEntry *__restrict__ sched, int 
 // with (i, j, k) the field node the extended node wraps to and i1, j1 the next node along
 // x and y (wrapped, or clamped on a closed axis).  The quads of u and v stand side by side in one
 // 32-byte record, those of w in a plane behind them, so a trilinear stencil is a 32-byte and a 16-byte
-// load for each of its two z-rows.  The L1 data stage bounds the advection: three 16-byte loads a row,
-// the quads of a node in one 48-byte run, kept it 94% busy (10.35 ms per 40 steps at 16.8M tracers on
-// 128^3 nodes, 400 steps 126.0 ms with the slices); the 32-byte loads take a fifth off its wavefronts
-// (80% busy, 10.08 ms, 124.4 ms), and the loads' latency at half the warps of an SM bounds what is left.
+// load for each of its two z-rows.  The L1 data stage bounds the advection: three 16-byte loads a row, the quads
+// of a node in one 48-byte run, take a fifth more of its wavefronts (400 steps of 16.8M tracers on 128^3 nodes, the
+// slices included, 126.0 ms; 124.4 with the 32-byte loads, the stage 76% busy on 64^3 nodes at the same density), and
+// the loads' latency at half the warps of an SM bounds what is left.
 // Stencil points a few cells outside the periodic box need no index wrapping: the halo holds the wrapped
 // values.
 //
@@ -398,8 +398,8 @@ __global__ void ep_slice_fill_kernel(RectParams P, SliceGeom G, const char *__re
 // stencil is eight 16-byte loads for the quads' two of 16 and two of 32, a slice a third of the bytes to write: for lattices
 // with few tracers per node, where writing the slices costs as much as reading them (slices_plain).  Two
 // x-neighbours in one 32-byte record (four loads, 32 bytes to write) was slower than nodes on sparse
-// lattices and than quads on dense ones (132.4 ms): at eight tracers per node every layout keeps the L1
-// data stage 90% busy, and this one returns a third more bytes than quads.
+// lattices and than quads on dense ones (132.4 ms): at eight tracers per node the L1 data stage
+// bounds every layout, and this one returns a third more bytes than quads.
 template <int ST>
 __global__ void __launch_bounds__(256) ep_node_fill_kernel(RectParams P, SliceGeom G, const char *__restrict__ pairs,
                                                            size_t fstride, const SchedEntry *__restrict__ stab,

@@ -1,4 +1,4 @@
-// mlp_gemm.cu -- BF16 GEMM on the tcgen05 tensor cores, used by the surrogate trainer.
+// mlp_gemm.cu -- BF16 GEMM on the tcgen05 tensor cores (lcs_gemm_bf16).
 //
 //   C[M x N] (+)= A[M x K] * B[N x K]^T      A, B: BF16, K contiguous; C: FP32
 //
