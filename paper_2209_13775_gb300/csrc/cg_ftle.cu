@@ -97,8 +97,10 @@ __device__ __forceinline__ AxisDiff axis_diff(const CgLaunch &L, const unsigned 
 }
 
 // F64: C, lambda_max or eigenpairs wanted (EIG: the latter), so grad F and C are formed in FP64 as well
+// The FTLE alone: four blocks per SM (64 registers; the positions stay live for the seeds that need FP64, which
+// would take 80 and leave three blocks: DP5(4) on 2.1M seeds with its FTLE, 3.295 -> 3.283 ms).
 template <int DIM, bool F64, bool EIG, int GM>
-__global__ void __launch_bounds__(256, EIG ? 3 : 1) cg_ftle_kernel(const __grid_constant__ CgLaunch L)
+__global__ void __launch_bounds__(256, EIG ? 3 : F64 ? 1 : 4) cg_ftle_kernel(const __grid_constant__ CgLaunch L)
 {
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int jr = blockIdx.y;        // job relative to job0
