@@ -112,7 +112,7 @@ __device__ __forceinline__ void mma_chain(uint32_t d, uint32_t a, uint32_t a_ste
 __global__ void __launch_bounds__(256, 1) train_step_kernel(const TrainArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint64_t bar_w, bar;
+    __shared__ uint64_t bar_w, bar, bar_end;
     __shared__ uint32_t tmem_base;
     __shared__ double red_l[4];
     __shared__ float red_g[4][3];
@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(256, 1) train_step_kernel(const TrainArgs A)
     if (tid == 0) {
         mbar_init(&bar_w, 1);
         mbar_init(&bar, 1);
+        mbar_init(&bar_end, 1);
         mbar_fence_init();
     }
     if (warp == 0) tmem_alloc(&tmem_base, 512);
@@ -134,8 +135,7 @@ __global__ void __launch_bounds__(256, 1) train_step_kernel(const TrainArgs A)
     for (int q = tid; q < 16 * TN / 8; q += 256) {    // rows 3..15 of dO stay zero
         *reinterpret_cast<uint4 *>(smem + DO_OFF + 16 * q) = make_uint4(0, 0, 0, 0);
     }
-    const bool have_w = !__syncthreads_or(!tc_wait(&bar_w, 0, A.errword, A.wait_ns));
-    bool ok = have_w;
+    bool ok = !__syncthreads_or(!tc_wait(&bar_w, 0, A.errword, A.wait_ns));
     const uint32_t tm = tmem_base, us = smem_u32(smem);
     const uint32_t tw = tm + TM_WORK + ((uint32_t)((warp & 3) * 32) << 16) + TH * g;   // this thread's lane and columns
     const float *bias = reinterpret_cast<const float *>(smem + BIAS_OFF);
@@ -377,12 +377,9 @@ __global__ void __launch_bounds__(256, 1) train_step_kernel(const TrainArgs A)
             for (int j = 0; j < 3; ++j) out[P_DB4 + j] = (red_g[0][j] + red_g[1][j]) + (red_g[2][j] + red_g[3][j]);
         }
     } else {
-        if (!have_w) {                                // a wait gave up: what is in flight ends first
-            mbar_wait_bounded(&bar_w, 0);
-        } else {
-            if (tid == 0) tc_commit(&bar);            // behind MMAs issued since the commit that was waited for
-            if (mbar_wait_bounded(&bar, phase ^ 1)) mbar_wait_bounded(&bar, phase);
-        }
+        mbar_wait_bounded(&bar_w, 0);                 // a wait gave up: what is in flight, the copy and all MMAs issued,
+        if (tid == 0) tc_commit(&bar_end);            // ends first
+        mbar_wait_bounded(&bar_end, 0);
         // nothing of an earlier batch is summed in this CTA's place, and the loss tells
         float4 *out = reinterpret_cast<float4 *>(A.part + (size_t)blockIdx.x * PART_STRIDE);
         for (int q = tid; q < PART_STRIDE / 4; q += 256) out[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
